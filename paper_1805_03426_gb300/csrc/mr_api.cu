@@ -382,12 +382,12 @@ void mr_destroy(mr_handle h)
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
     DeviceBuffers& b = h->buf;
-    void* ptrs[] = {b.T[0], b.T[1], b.T[2], b.U64, b.V64, b.W64, b.Us, b.Vs, b.Ws, b.scrW, b.scrV,
+    void* ptrs[] = {b.T[0], b.T[1], b.T[2], b.U64, b.V64, b.W64, b.Us, b.Vs, b.Ws, b.vmax, b.scrW, b.scrV,
                     b.metric, b.red, b.nu2, b.stage, b.tri};
     for (void* p : ptrs)
         if (p) dev_free(p);
     DeviceBuffers::Level& n = b.next;
-    void* nptrs[] = {n.U64, n.V64, n.W64, n.Us, n.Vs, n.Ws, n.xwy, n.xuo, n.xvr, b.lerpc};
+    void* nptrs[] = {n.U64, n.V64, n.W64, n.Us, n.Vs, n.Ws, n.vmax, n.xwy, n.xuo, n.xvr, b.lerpc};
     for (void* p : nptrs)
         if (p) dev_free(p);
     if (h->elt == 4) {
@@ -494,6 +494,7 @@ int mr_create(const mr_config* cfg, mr_handle* out)
         alloc(&b.Us, h->nU * h->elt);
         alloc(&b.Vs, h->nV * h->elt);
         alloc(&b.Ws, h->nW * h->elt);
+        if (h->elt == 8) alloc((void**)&b.vmax, 4 * sizeof(unsigned));
         alloc(&b.scrW, (size_t)(h->Nz + 1) * c.ny * c.nx * h->elt);
         alloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * c.nx * h->elt);
     }
@@ -705,8 +706,24 @@ static int derive_velocity(mr_handle h, bool convert, cudaStream_t st)
                                          h->cfg.nx, h->cfg.ny, h->cfg.nz, h->slab ? h->cfg.slab_j0 : 0, h->nys, st);
         if (e != cudaSuccess) return cuda_check(e, "padded coarse faces");
     }
-    if (h->cfg.velocity_mode == MR_VEL_STORED) return refine_into(h, b.Us, b.Vs, b.Ws, st);
+    if (h->cfg.velocity_mode == MR_VEL_STORED) {
+        const int rc = refine_into(h, b.Us, b.Vs, b.Ws, st);
+        if (rc || !b.vmax) return rc;
+        return cuda_check(launch_vmax((const double*)b.Us, h->nU, (const double*)b.Vs, h->nV, (const double*)b.Ws,
+                                      h->nW, b.vmax, st), "velocity maxima");
+    }
     return MR_OK;
+}
+
+// One step of the scalar on the handle's dense FP64 faces (the explicit part, with
+// implicit vertical diffusion): in fixed point where the grid fits.
+static cudaError_t step_f64(mr_handle h, const double* Tm1, const double* T, double* Tp1, StepCoef c, cudaStream_t st)
+{
+    const DeviceBuffers& b = h->buf;
+    const double *u = (const double*)b.Us, *v = (const double*)b.Vs, *w = (const double*)b.Ws;
+    const bool implz = h->cfg.diffz_implicit != 0;
+    if (step_fix_fits(h->g64)) return launch_step_fix(h->g64, u, v, w, Tm1, T, Tp1, c, implz, b.vmax, st);
+    return launch_step_stored<double>(h->g64, u, v, w, Tm1, T, Tp1, c, implz, st);
 }
 
 // One time step of the scalar.  alpha = 0: the current velocity; otherwise the
@@ -726,8 +743,7 @@ static int one_step(mr_handle h, double alpha, cudaStream_t st, double* Tc = nul
         const double* B[3] = {(const double*)nx.Us, (const double*)nx.Vs, (const double*)nx.Ws};
         e = lerp ? launch_step_stored_lerp<double>(h->g64, A, B, alpha, (const double*)Tm1, (const double*)b.T[h->ic],
                                                    (double*)b.T[in], c, implz, st)
-                 : launch_step_stored<double>(h->g64, A[0], A[1], A[2], (const double*)Tm1, (const double*)b.T[h->ic],
-                                              (double*)b.T[in], c, implz, st);
+                 : step_f64(h, (const double*)Tm1, (const double*)b.T[h->ic], (double*)b.T[in], c, st);
         if (e == cudaSuccess && implz) e = launch_zsolve<double>(h->g64, (double*)b.T[in], 0.5 * c.gdt, (double*)b.tri, st);
     } else if (h->cfg.velocity_mode == MR_VEL_XFUSED) {
         const float* A[3] = {b.xwy, b.xuo, b.xvr};
@@ -787,6 +803,7 @@ static void swap_levels(DeviceBuffers& b)
     std::swap(b.U64, n.U64); std::swap(b.V64, n.V64); std::swap(b.W64, n.W64);
     std::swap(b.Uc, n.Uc); std::swap(b.Vc, n.Vc); std::swap(b.Wc, n.Wc);
     std::swap(b.Us, n.Us); std::swap(b.Vs, n.Vs); std::swap(b.Ws, n.Ws);
+    std::swap(b.vmax, n.vmax);
     std::swap(b.xwy, n.xwy); std::swap(b.xuo, n.xuo); std::swap(b.xvr, n.xvr);
     std::swap(b.cpad, n.cpad);
 }
@@ -814,6 +831,7 @@ static int alloc_next(mr_handle h)
         alloc(&n.Us, h->nU * h->elt);
         alloc(&n.Vs, h->nV * h->elt);
         alloc(&n.Ws, h->nW * h->elt);
+        if (h->elt == 8) alloc((void**)&n.vmax, 4 * sizeof(unsigned));
     } else if (mode == MR_VEL_XFUSED) {
         alloc((void**)&n.xwy, (size_t)(h->Nz + 1) * h->Ny * b.nxg * 4);
         alloc((void**)&n.xuo, (size_t)h->Nz * h->Ny * b.nxg * 4);
@@ -824,7 +842,7 @@ static int alloc_next(mr_handle h)
         alloc((void**)&b.lerpc, np * 4);
     }
     if (e != cudaSuccess) {
-        void* ptrs[] = {n.U64, n.V64, n.W64, n.Us, n.Vs, n.Ws, n.xwy, n.xuo, n.xvr, n.cpad, b.lerpc};
+        void* ptrs[] = {n.U64, n.V64, n.W64, n.Us, n.Vs, n.Ws, n.vmax, n.xwy, n.xuo, n.xvr, n.cpad, b.lerpc};
         for (void* p : ptrs)
             if (p) dev_free(p);
         if (h->elt == 4) {
@@ -1335,8 +1353,7 @@ cudaError_t step_buffers(mr_handle h, const void* Tm1, const void* T, void* Tp1,
     const void* tm = s == 0 ? T : Tm1;
     const DeviceBuffers& b = h->buf;
     if (h->cfg.precision == MR_F64)
-        return launch_step_stored<double>(h->g64, (const double*)b.Us, (const double*)b.Vs, (const double*)b.Ws,
-                                          (const double*)tm, (const double*)T, (double*)Tp1, c, false, st);
+        return step_f64(h, (const double*)tm, (const double*)T, (double*)Tp1, c, st);
     return launch_step_stored<float>(h->g32, (const float*)b.Us, (const float*)b.Vs, (const float*)b.Ws,
                                      (const float*)tm, (const float*)T, (float*)Tp1, c, false, st);
 }

@@ -1,0 +1,80 @@
+// 64-bit fixed-point arithmetic on the integer pipes, for the FP64 path.
+//
+// GB300 issues FP64 arithmetic (and every conversion from or to FP64) at 2
+// lanes per clock and SM, 1/64 of its FP32 rate, but 32 x 32 + 64-bit integer
+// multiply-adds at ~50 and 32-bit integer operations at 64 lanes per clock and
+// SM (measured).  So a stencil over values of one scale is several times faster
+// in integers: every value becomes a 60- or 62-bit integer relative to the
+// largest one of its neighbourhood, sums of integers are exact, and a product
+// of two of them is three multiply-adds of balanced 32-bit halves with an error
+// of 2^-60 of its largest value, where FP64 rounds at 2^-53 of its own.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace mr {
+namespace fix {
+
+// x = hi 2^32 + lo with both halves signed
+struct Bal {
+    int hi, lo;
+};
+__host__ __device__ __forceinline__ Bal bal(long long x)
+{
+    const unsigned lo = (unsigned)x;
+    return {(int)(x >> 32) + (int)(lo >> 31), (int)lo};
+}
+
+// a sum of products: H 2^64 + M 2^32 (the products of the low halves are left out)
+struct Acc {
+    long long H, M;
+};
+__host__ __device__ __forceinline__ long long madw(int a, int b, long long c)
+{
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+#else
+    return (long long)a * b + c;
+#endif
+}
+__host__ __device__ __forceinline__ void mac(Acc& s, Bal a, Bal b)
+{
+    s.M = madw(a.hi, b.lo, s.M);
+    s.M = madw(a.lo, b.hi, s.M);
+    s.H = madw(a.hi, b.hi, s.H);
+}
+// the product in units of 2^64
+__host__ __device__ __forceinline__ long long mul(Bal a, Bal b)
+{
+    Acc s{0, 0};
+    mac(s, a, b);
+    return madw((int)(s.M >> 32), 1, s.H);
+}
+
+// The double with words (hi, lo) as an integer of at most BITS bits relative to
+// the exponent field E >= its own: trunc(|x| 2^(BITS - (E - 1022))), the sign by
+// complement (so negative values come out one unit lower).  Zeros and
+// subnormals, whose field is 0, come out as 0 (or -1) for every E >= 80.
+template <int BITS>
+__host__ __device__ __forceinline__ long long dec(int hi, int lo, int E)
+{
+    constexpr int L = BITS - 53;
+    // E - e from the magnitude's high word, which a caller may have taken already
+    const int d = (int)((((unsigned)E << 20) | 0xfffffu) - ((unsigned)hi & 0x7fffffffu)) >> 20;
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u, ml = (unsigned)lo;
+    const int s = hi >> 31;
+#ifdef __CUDA_ARCH__
+    const unsigned long long m = ((unsigned long long)__funnelshift_l(ml, mh, L) << 32) | (ml << L);
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(d));       // 0 from 64 on
+#else
+    const unsigned long long m = ((unsigned long long)mh << 32 | ml) << L, r = d > 63 ? 0ull : m >> d;
+#endif
+    return (long long)((unsigned long long)(unsigned)((int)(r >> 32) ^ s) << 32 | (unsigned)((int)r ^ s));
+}
+
+}  // namespace fix
+}  // namespace mr

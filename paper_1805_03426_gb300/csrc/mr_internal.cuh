@@ -68,6 +68,7 @@ struct DeviceBuffers {
     void* Us = nullptr;                        // dense faces (MR_VEL_STORED)
     void* Vs = nullptr;
     void* Ws = nullptr;
+    unsigned* vmax = nullptr;                  // MR_VEL_STORED, FP64: largest |U|, |V|, |W| (high words)
     void* scrW = nullptr;                      // refinement scratch: full-coarse-area W per dense plane
     void* scrV = nullptr;                      // refinement scratch: full-coarse-width V per dense row
     void* metric = nullptr;                    // one block holding every Grid array
@@ -99,6 +100,7 @@ struct DeviceBuffers {
         double *U64 = nullptr, *V64 = nullptr, *W64 = nullptr;
         void *Uc = nullptr, *Vc = nullptr, *Wc = nullptr;
         void *Us = nullptr, *Vs = nullptr, *Ws = nullptr;
+        unsigned* vmax = nullptr;
         float *xwy = nullptr, *xuo = nullptr, *xvr = nullptr;
         float* cpad = nullptr;
     } next;
@@ -172,6 +174,14 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
 template <typename P>
 cudaError_t launch_step_stored(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, const P* Tm1,
                                const P* T, P* Tp1, StepCoef c, bool implz, cudaStream_t st);
+// the FP64 step in 64-bit fixed point (mr_step64.cu), the grids it takes, and the
+// largest magnitudes of the velocity components that it needs
+bool step_fix_fits(const Grid<double>& g);
+cudaError_t launch_step_fix(const Grid<double>& g, const double* Us, const double* Vs, const double* Ws,
+                            const double* Tm1, const double* T, double* Tp1, StepCoef c, bool implz,
+                            const unsigned* vmax, cudaStream_t st);
+cudaError_t launch_vmax(const double* U, size_t nU, const double* V, size_t nV, const double* W, size_t nW,
+                        unsigned* vmax, cudaStream_t st);
 // the same step with the velocity A + alpha (B - A) of two stored dense fields
 template <typename P>
 cudaError_t launch_step_stored_lerp(const Grid<P>& g, const P* const velA[3], const P* const velB[3], double alpha,
