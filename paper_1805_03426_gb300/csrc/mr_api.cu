@@ -248,6 +248,8 @@ static int upload_metric(mr_handle_s* h, char* dst, const int* dwin, Grid<P>& g)
         cdn[k] = (k > 0 || dir) ? h->kappa / (h->dz[k] * below) : 0.0;
         cup[k] = (k < Nz - 1 || dir) ? h->kappa / (h->dz[k] * above) : 0.0;
     }
+    h->cdn = cdn;
+    h->cup = cup;
     const double dx = c.lx / h->Nx, dy = c.ly / h->Ny;
     const double kx2 = h->kappa / (dx * dx), ky2 = h->kappa / (dy * dy);
     std::vector<double> lz(8 * (size_t)Nz);
@@ -507,7 +509,7 @@ int mr_create(const mr_config* cfg, mr_handle* out)
     if (e == cudaSuccess) e = cudaMemset(b.nu2, 0, (3 + 2 * kPlateBlocks) * sizeof(double));   // the block count
     h->stage_bytes = std::min<size_t>((size_t)64 << 20, std::max<size_t>(h->ncell * 8, 1 << 16));
     alloc(&b.stage, h->stage_bytes);
-    if (c.diffz_implicit) alloc(&b.tri, h->ncell * h->elt);
+    if (c.diffz_implicit && zsolve_needs_work(h->Nz)) alloc(&b.tri, h->ncell * h->elt);
     if (c.velocity_mode == MR_VEL_XFUSED) {
         b.nxg = c.nx + 8;
         alloc((void**)&b.xwy, (size_t)(h->Nz + 1) * h->Ny * b.nxg * 4);
@@ -744,7 +746,7 @@ static int one_step(mr_handle h, double alpha, cudaStream_t st, double* Tc = nul
         e = lerp ? launch_step_stored_lerp<double>(h->g64, A, B, alpha, (const double*)Tm1, (const double*)b.T[h->ic],
                                                    (double*)b.T[in], c, implz, st)
                  : step_f64(h, (const double*)Tm1, (const double*)b.T[h->ic], (double*)b.T[in], c, st);
-        if (e == cudaSuccess && implz) e = launch_zsolve<double>(h->g64, (double*)b.T[in], 0.5 * c.gdt, (double*)b.tri, st);
+        if (e == cudaSuccess && implz) e = launch_zsolve<double>(h->g64, (double*)b.T[in], 0.5 * c.gdt, h->cdn.data(), h->cup.data(), (double*)b.tri, st);
     } else if (h->cfg.velocity_mode == MR_VEL_XFUSED) {
         const float* A[3] = {b.xwy, b.xuo, b.xvr};
         const float* B[3] = {nx.xwy, nx.xuo, nx.xvr};
@@ -786,7 +788,7 @@ static int one_step(mr_handle h, double alpha, cudaStream_t st, double* Tc = nul
                                                   (float*)b.T[in], c, implz, st)
                  : launch_step_stored<float>(h->g32, A[0], A[1], A[2], (const float*)Tm1, (const float*)b.T[h->ic],
                                              (float*)b.T[in], c, implz, st);
-        if (e == cudaSuccess && implz) e = launch_zsolve<float>(h->g32, (float*)b.T[in], 0.5 * c.gdt, (float*)b.tri, st);
+        if (e == cudaSuccess && implz) e = launch_zsolve<float>(h->g32, (float*)b.T[in], 0.5 * c.gdt, h->cdn.data(), h->cup.data(), (float*)b.tri, st);
     }
     if (e != cudaSuccess) return cuda_check(e, "scalar step launch");
     h->ip = h->ic;

@@ -75,7 +75,7 @@ struct DeviceBuffers {
     double* red = nullptr;                     // reduction partials
     double* nu2 = nullptr;                     // plate Nusselt numbers (2 doubles + partials)
     void* stage = nullptr;                     // conversion staging buffer
-    void* tri = nullptr;                       // implicit-z work (2 * Nz per column)
+    void* tri = nullptr;                       // implicit-z work of tall columns (zsolve_needs_work)
     // MR_VEL_XFUSED: coarse-x intermediates of the z- and y-stages (FP32,
     // nxg = nx + 8 columns with 4 periodic ghosts each side) and layer constants
     float* xwy = nullptr;                      // [Nz+1][Ny][nxg]
@@ -135,7 +135,7 @@ struct mr_handle_s {
     bool maxdiv_valid = false;
     double maxdiv = 0.0;
     // host FP64 grid (Section 3.1) and R matrices (Section 3.2)
-    std::vector<double> zf, zc, dz, Rx, Ry, Rz;
+    std::vector<double> zf, zc, dz, cdn, cup, Rx, Ry, Rz;
     std::vector<double> f4x, f4y, f4z;   // fourth-order face weights (zeros at face_order 2)
     std::vector<int> wx, wy, wz;
     mr::DeviceBuffers buf;
@@ -189,7 +189,9 @@ cudaError_t launch_step_stored_lerp(const Grid<P>& g, const P* const velA[3], co
 // out = A + alpha (B - A), elementwise (coarse faces of two time levels)
 cudaError_t launch_lerp_f32(const float* A, const float* B, double alpha, float* out, size_t n, cudaStream_t st);
 template <typename P>
-cudaError_t launch_zsolve(const Grid<P>& g, P* Tp1, double half_gdt, P* work, cudaStream_t st);
+cudaError_t launch_zsolve(const Grid<P>& g, P* Tp1, double half_gdt, const double* cdn, const double* cup, P* work,
+                          cudaStream_t st);
+bool zsolve_needs_work(int Nz);   // whether launch_zsolve uses work (one value per cell)
 template <typename P>
 cudaError_t launch_convert(const void* src, int src_dtype, void* dst, int dst_dtype, size_t n,
                            cudaStream_t st);

@@ -165,10 +165,87 @@ __global__ void __launch_bounds__(256) k_step_periodic(Grid<P> g, const P* __res
 
 // Opt-in implicit vertical diffusion: per (x, y) column solve
 //   (1 + h (cup + cdn)) x_k - h cdn_k x_{k-1} - h cup_k x_{k+1} = r_k,
-// h = gdt / 2, by the Thomas algorithm; work holds the eliminated
-// super-diagonal (one value per cell).
+// h = gdt / 2, by elimination from both plates at once: lanes 0..15 of a warp
+// eliminate the lower halves of 16 columns upwards, lanes 16..31 their upper
+// halves downwards, the two middle values follow from one exchange, and both
+// substitute back towards their plate.  The eliminated coefficients do not
+// depend on the column, so the host forms them (ZTable, in FP64) and they come
+// with the launch: per layer, counted from the lane's plate,
+//   y_n = id r_n + e y_{n-1},   then   x_n = y_n + f x_{n+1},
+// three multiply-adds per cell and no division.  The loads of eight layers are
+// in flight ahead of the chain, and y stays in shared memory where a block's
+// columns fit (SM), so that X is read and written once; blocks of one warp
+// spread the columns over the SMs.  What bounds it is the FP64 pipe, which takes
+// 64 clocks per instruction of a warp, so half the layers per warp on twice the
+// warps is what fills the chip's pipes on small planes.
+// Measured on 123 x 74 x 148 cells in FP64 (ncu): 19.4 us; 29.7 us with a whole
+// column per lane, 224 us with two FP64 divisions per cell and the coefficients
+// in global memory.
+constexpr int kZBatch = 8;
+template <typename P, int N>
+struct ZTable {
+    P id[N], e[N], f[N];
+    P mid;                                                 // 1 / (1 - f f) of the middle pair
+};
+template <typename P, int N, bool SM>
+__global__ void __launch_bounds__(32) k_zsolve(P* __restrict__ X, size_t plane, int Nz,
+                                               const __grid_constant__ ZTable<P, N> z)
+{
+    extern __shared__ __align__(16) unsigned char zsm[];
+    const int lane = threadIdx.x;
+    const bool up = lane >= 16;                            // from the upper plate
+    const size_t m = (size_t)blockIdx.x * 16 + (lane & 15);
+    const bool on = m < plane;                             // off: a column of the domain, read but not written
+    P* const x = X + (on ? m : plane - 1) + (up ? (size_t)(Nz - 1) * plane : 0);
+    const ptrdiff_t step = up ? -(ptrdiff_t)plane : (ptrdiff_t)plane;
+    const int cnt = up ? Nz - Nz / 2 : Nz / 2, k0 = up ? Nz - 1 : 0, dk = up ? -1 : 1;
+    P* const y = reinterpret_cast<P*>(zsm) + lane;
+    P r[kZBatch], v = P(0);
+#pragma unroll
+    for (int q = 0; q < kZBatch; ++q) r[q] = q < cnt ? x[q * step] : P(0);
+    for (int n0 = 0; n0 < cnt; n0 += kZBatch) {
+        P c[kZBatch];
+#pragma unroll
+        for (int q = 0; q < kZBatch; ++q) {
+            c[q] = r[q];
+            const int n = n0 + kZBatch + q;
+            if (n < cnt) r[q] = x[n * step];
+        }
+#pragma unroll
+        for (int q = 0; q < kZBatch; ++q) {
+            const int n = n0 + q, k = k0 + n * dk;
+            if (n < cnt) {
+                v = z.id[k] * c[q] + z.e[k] * v;
+                if (SM) y[n * 32] = v;
+                else if (on) x[n * step] = v;
+            }
+        }
+    }
+    __syncwarp();
+    // the middle pair: x = y + f x_other on both sides
+    const P vo = __shfl_xor_sync(0xffffffffu, v, 16);
+    if (cnt == 0) return;
+    v = (v + z.f[k0 + (cnt - 1) * dk] * vo) * z.mid;
+    if (on) x[(cnt - 1) * step] = v;
+    for (int n0 = cnt - 2; n0 >= 0; n0 -= kZBatch) {
+        P c[kZBatch];
+#pragma unroll
+        for (int q = 0; q < kZBatch; ++q) c[q] = n0 - q >= 0 ? (SM ? y[(n0 - q) * 32] : x[(n0 - q) * step]) : P(0);
+#pragma unroll
+        for (int q = 0; q < kZBatch; ++q) {
+            const int n = n0 - q;
+            if (n >= 0) {
+                v = c[q] + z.f[k0 + n * dk] * v;
+                if (on) x[n * step] = v;
+            }
+        }
+    }
+}
+
+// The same for columns whose coefficients exceed a launch's parameters: formed
+// per column, the eliminated super-diagonal in work (one value per cell).
 template <typename P>
-__global__ void k_zsolve(Grid<P> g, P* __restrict__ X, P h, P* __restrict__ work)
+__global__ void k_zsolve_tall(Grid<P> g, P* __restrict__ X, P h, P* __restrict__ work)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
@@ -193,6 +270,44 @@ __global__ void k_zsolve(Grid<P> g, P* __restrict__ X, P h, P* __restrict__ work
         prev_x = X[base + k * plane] - work[base + k * plane] * prev_x;
         X[base + k * plane] = prev_x;
     }
+}
+
+template <typename P, int N>
+cudaError_t zsolve_table(const Grid<P>& g, P* X, double h, const double* cdn, const double* cup, cudaStream_t st)
+{
+    ZTable<P, N> z;
+    const int M = g.Nz / 2;                                // layers of the lower half
+    double c = 0.0, fb = 0.0, ft = 0.0;                    // what the layer nearer to the plate left on this one
+    for (int k = 0; k < M; ++k) {
+        const double lo = k > 0 ? h * cdn[k] : 0.0, id = 1.0 / (1.0 + h * (cup[k] + cdn[k]) - lo * c);
+        c = (k < g.Nz - 1 ? h * cup[k] : 0.0) * id;
+        z.id[k] = (P)id;
+        z.e[k] = (P)(lo * id);
+        z.f[k] = (P)(fb = c);
+    }
+    c = 0.0;
+    for (int k = g.Nz - 1; k >= M; --k) {
+        const double up = k < g.Nz - 1 ? h * cup[k] : 0.0, id = 1.0 / (1.0 + h * (cup[k] + cdn[k]) - up * c);
+        c = (k > 0 ? h * cdn[k] : 0.0) * id;
+        z.id[k] = (P)id;
+        z.e[k] = (P)(up * id);
+        z.f[k] = (P)(ft = c);
+    }
+    z.mid = (P)(1.0 / (1.0 - fb * ft));
+    const size_t plane = (size_t)g.Nx * g.Ny;
+    const unsigned blocks = (unsigned)((plane + 15) / 16);
+    const int bytes = (g.Nz - M) * 32 * (int)sizeof(P);
+    // at least four blocks of one warp per SM (one per scheduler); beyond that y goes
+    // through global memory
+    if (bytes <= 56 * 1024) {
+        static unsigned long long done = 0;                // one bit per device
+        const cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_zsolve<P, N, true>), 56 * 1024, &done);
+        if (e != cudaSuccess) return e;
+        k_zsolve<P, N, true><<<blocks, 32, bytes, st>>>(X, plane, g.Nz, z);
+    } else {
+        k_zsolve<P, N, false><<<blocks, 32, 0, st>>>(X, plane, g.Nz, z);
+    }
+    return cudaGetLastError();
 }
 
 template <typename P, bool LERP>
@@ -257,12 +372,19 @@ cudaError_t launch_step_stored_lerp(const Grid<P>& g, const P* const velA[3], co
                                 T, Tp1, c, implz, st);
 }
 
+// The largest table is 3 x 1280 doubles (30 KB of the 32,764 bytes of parameters a
+// launch may have); the small one keeps the usual launches short.
+bool zsolve_needs_work(int Nz) { return Nz > 1280; }
+
 template <typename P>
-cudaError_t launch_zsolve(const Grid<P>& g, P* Tp1, double half_gdt, P* work, cudaStream_t st)
+cudaError_t launch_zsolve(const Grid<P>& g, P* Tp1, double half_gdt, const double* cdn, const double* cup, P* work,
+                          cudaStream_t st)
 {
+    if (g.Nz <= 256) return zsolve_table<P, 256>(g, Tp1, half_gdt, cdn, cup, st);
+    if (!zsolve_needs_work(g.Nz)) return zsolve_table<P, 1280>(g, Tp1, half_gdt, cdn, cup, st);
     dim3 blk(128);
     dim3 grd((g.Nx + 127) / 128, g.Ny);
-    k_zsolve<P><<<grd, blk, 0, st>>>(g, Tp1, (P)half_gdt, work);
+    k_zsolve_tall<P><<<grd, blk, 0, st>>>(g, Tp1, (P)half_gdt, work);
     return cudaGetLastError();
 }
 
@@ -278,7 +400,9 @@ template cudaError_t launch_step_stored_lerp<double>(const Grid<double>&, const 
 template cudaError_t launch_step_stored_lerp<float>(const Grid<float>&, const float* const[3], const float* const[3],
                                                     double, const float*, const float*, float*, StepCoef, bool,
                                                     cudaStream_t);
-template cudaError_t launch_zsolve<double>(const Grid<double>&, double*, double, double*, cudaStream_t);
-template cudaError_t launch_zsolve<float>(const Grid<float>&, float*, double, float*, cudaStream_t);
+template cudaError_t launch_zsolve<double>(const Grid<double>&, double*, double, const double*, const double*, double*,
+                                           cudaStream_t);
+template cudaError_t launch_zsolve<float>(const Grid<float>&, float*, double, const double*, const double*, float*,
+                                          cudaStream_t);
 
 }  // namespace mr
