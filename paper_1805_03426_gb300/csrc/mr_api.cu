@@ -385,7 +385,7 @@ void mr_destroy(mr_handle h)
     cudaDeviceSynchronize();
     DeviceBuffers& b = h->buf;
     void* ptrs[] = {b.T[0], b.T[1], b.T[2], b.U64, b.V64, b.W64, b.Us, b.Vs, b.Ws, b.vmax, b.scrW, b.scrV,
-                    b.metric, b.red, b.nu2, b.stage, b.tri};
+                    b.metric, b.red, b.mom, b.prof, b.nu2, b.stage, b.tri};
     for (void* p : ptrs)
         if (p) dev_free(p);
     DeviceBuffers::Level& n = b.next;
@@ -502,9 +502,11 @@ int mr_create(const mr_config* cfg, mr_handle* out)
     }
     const size_t mb64 = metric_bytes<double>(h), mb32 = metric_bytes<float>(h);
     const size_t nwin = 3 * ((size_t)c.nx + c.ny + c.nz);
-    alloc(&b.metric, mb64 + mb32 + nwin * sizeof(int));
+    alloc(&b.metric, mb64 + mb32 + (size_t)h->Nz * sizeof(double) + nwin * sizeof(int));
     h->red_blocks = 152 * 8;
     alloc((void**)&b.red, (size_t)h->red_blocks * 2 * sizeof(double));
+    alloc((void**)&b.mom, (1 + 6 * (size_t)kMomentBlocks + 8) * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemset(b.mom, 0, (1 + 6 * (size_t)kMomentBlocks + 8) * sizeof(double));
     alloc((void**)&b.nu2, (3 + 2 * kPlateBlocks) * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(b.nu2, 0, (3 + 2 * kPlateBlocks) * sizeof(double));   // the block count
     h->stage_bytes = std::min<size_t>((size_t)64 << 20, std::max<size_t>(h->ncell * 8, 1 << 16));
@@ -532,8 +534,17 @@ int mr_create(const mr_config* cfg, mr_handle* out)
     win.insert(win.end(), h->wx.begin(), h->wx.end());
     win.insert(win.end(), h->wy.begin(), h->wy.end());
     win.insert(win.end(), h->wz.begin(), h->wz.end());
-    int* dwin = (int*)((char*)b.metric + mb64 + mb32);
-    e = cudaMemcpy(dwin, win.data(), win.size() * sizeof(int), cudaMemcpyHostToDevice);
+    // upscale weights (FP64), then the windows, behind the two metrics
+    std::vector<double> upw(h->Nz);
+    for (int K = 0; K < c.nz; ++K) {
+        double z = 0.0;
+        for (int k = K * c.mz; k < (K + 1) * c.mz; ++k) z += h->dz[k];
+        for (int k = K * c.mz; k < (K + 1) * c.mz; ++k) upw[k] = h->dz[k] / (z * c.mx * c.my);
+    }
+    b.upw = (const double*)((char*)b.metric + mb64 + mb32);
+    int* dwin = (int*)(b.upw + h->Nz);
+    e = cudaMemcpy((void*)b.upw, upw.data(), upw.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(dwin, win.data(), win.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         int r = cuda_check(e, "mr_create: upload windows");
         mr_destroy(h);
@@ -1109,8 +1120,8 @@ int mr_scalar_step_coupled(mr_handle h, double* nu2, double* Tc, mr_stream strea
             if (e == cudaSuccess) e = cudaMemcpyAsync(dnu, h->buf.nu2, 2 * sizeof(double), cudaMemcpyDefault, st);
         }
         if (e == cudaSuccess && dtc)
-            e = h->cfg.precision == MR_F64 ? launch_upscale<double>(h->g64, (const double*)h->buf.T[h->ic], dtc, st)
-                                           : launch_upscale<float>(h->g32, (const float*)h->buf.T[h->ic], dtc, st);
+            e = h->cfg.precision == MR_F64 ? launch_upscale<double>(h->g64, (const double*)h->buf.T[h->ic], h->buf.upw, dtc, st)
+                                           : launch_upscale<float>(h->g32, (const float*)h->buf.T[h->ic], h->buf.upw, dtc, st);
     }
     return cuda_check(e, "mr_scalar_step_coupled");
 }
@@ -1158,36 +1169,55 @@ int mr_plate_nu(mr_handle h, double* nu2, mr_stream stream)
     return cuda_check(cudaMemcpyAsync(nu2, h->buf.nu2, 2 * sizeof(double), cudaMemcpyDefault, st), "mr_plate_nu: copy");
 }
 
-static int reduce_partials(mr_handle h, int nper, std::vector<double>& out, cudaStream_t st)
+// Launch the maximum over the dense cells of |divergence| (kind 1) or of the CFL
+// rate (kind 2) of the refined velocity: partials in buf.red, *n of them.
+static cudaError_t launch_velocity_max(mr_handle h, int kind, int* n, cudaStream_t st)
 {
-    out.resize((size_t)h->red_blocks * nper);
-    cudaError_t e = cudaMemcpyAsync(out.data(), h->buf.red, out.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return cuda_check(e, "reduction");
+    const DeviceBuffers& b = h->buf;
+    *n = 1;
+    if (h->cfg.velocity_mode == MR_VEL_XFUSED)
+        return launch_xfused_max_f32(h->g32, kind, b.xwy, b.xuo, b.xvr, b.nxg, b.xlc, b.xlcw, b.xrx, b.red, 1, st);
+    if (h->cfg.velocity_mode == MR_VEL_FUSED)
+        return launch_fused_max_f32(h->g32, kind, FusedInputs{b.cpad, {}, {}, 0, b.fsc, b.xlc, b.xrx, b.xry, nullptr, nullptr},
+                                    b.red, 1, st);
+    *n = h->red_blocks;
+    if (h->cfg.precision == MR_F64) {
+        const double *u = (const double*)b.Us, *v = (const double*)b.Vs, *w = (const double*)b.Ws;
+        return kind == 1 ? launch_maxdiv<double>(h->g64, u, v, w, b.red, *n, st)
+                         : launch_cfl<double>(h->g64, u, v, w, b.red, *n, st);
+    }
+    const float *u = (const float*)b.Us, *v = (const float*)b.Vs, *w = (const float*)b.Ws;
+    return kind == 1 ? launch_maxdiv<float>(h->g32, u, v, w, b.red, *n, st) : launch_cfl<float>(h->g32, u, v, w, b.red, *n, st);
 }
 
-static int max_divergence(mr_handle h, double* out, cudaStream_t st)
+// The stored cells' volume over dx dy.
+static double column_volume(mr_handle h)
 {
-    cudaError_t e;
-    const DeviceBuffers& b = h->buf;
-    if (h->cfg.velocity_mode == MR_VEL_XFUSED)
-        e = launch_xfused_max_f32(h->g32, 1, b.xwy, b.xuo, b.xvr, b.nxg, b.xlc, b.xlcw, b.xrx, b.red, h->red_blocks, st);
-    else if (h->cfg.velocity_mode == MR_VEL_FUSED)
-        e = launch_fused_max_f32(h->g32, 1, FusedInputs{b.cpad, {}, {}, 0, b.fsc, b.xlc, b.xrx, b.xry, nullptr, nullptr}, b.red,
-                                 h->red_blocks, st);
-    else if (h->cfg.precision == MR_F64)
-        e = launch_maxdiv<double>(h->g64, (const double*)b.Us, (const double*)b.Vs, (const double*)b.Ws, b.red,
-                                  h->red_blocks, st);
-    else
-        e = launch_maxdiv<float>(h->g32, (const float*)b.Us, (const float*)b.Vs, (const float*)b.Ws, b.red,
-                                 h->red_blocks, st);
-    if (e != cudaSuccess) return cuda_check(e, "max divergence: launch");
-    std::vector<double> p;
-    int rc = reduce_partials(h, 1, p, st);
-    if (rc) return rc;
-    double m = 0.0;
-    for (double v : p) m = std::max(m, v);
-    *out = m;
+    double v = 0.0;
+    for (int k = 0; k < h->Nz; ++k) v += h->dz[k];
+    return v * (double)h->Nx * (double)h->Nys;
+}
+
+// Volume moments of a dense field in the handle's precision into the handle's results.
+static cudaError_t launch_field_moments(mr_handle h, const void* T, cudaStream_t st)
+{
+    double* const res = h->buf.mom + 1 + 6 * (size_t)kMomentBlocks;
+    return h->cfg.precision == MR_F64
+               ? launch_moments<double>(h->g64, (const double*)T, h->g64.dz, column_volume(h), h->buf.mom, res, st)
+               : launch_moments<float>(h->g32, (const float*)T, h->g64.dz, column_volume(h), h->buf.mom, res, st);
+}
+
+// Gather what was launched (launch_gather) and bring the handle's eight results
+// to the host: one small copy and one synchronisation.
+static int take_results(mr_handle h, bool nu, int nmax, double res[8], cudaStream_t st, const char* what)
+{
+    double* const dres = h->buf.mom + 1 + 6 * (size_t)kMomentBlocks;
+    int* const err = h->cfg.velocity_mode != MR_VEL_STORED ? fused_error_peek() : nullptr;
+    cudaError_t e = launch_gather(nu ? h->buf.nu2 : nullptr, nmax ? h->buf.red : nullptr, nmax, err, dres, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(res, dres, 8 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_check(e, what);
+    if (res[6] != 0.0) return set_error(MR_ERR_TIMEOUT, std::string(what) + ": a fused kernel gave up a bounded wait");
     return MR_OK;
 }
 
@@ -1196,47 +1226,33 @@ int mr_scalar_stats(mr_handle h, mr_stats* out, mr_stream stream)
     if (!h || !out) return set_error(MR_ERR_ARG, "mr_scalar_stats: NULL argument");
     if (!h->have_scalar) return set_error(MR_ERR_STATE, "mr_scalar_stats: no scalar set");
     cudaStream_t st = (cudaStream_t)stream;
-    if (h->cfg.velocity_mode != MR_VEL_STORED && fused_take_error(st) == MR_ERR_TIMEOUT)
-        return set_error(MR_ERR_TIMEOUT, "mr_scalar_stats: a fused step kernel gave up a bounded wait");
     const void* T = h->buf.T[h->ic];
-    const double dxdy = (h->cfg.lx / h->Nx) * (h->cfg.ly / h->Ny);
-    double vtot = 0.0;
-    for (int k = 0; k < h->Nz; ++k) vtot += h->dz[k];
-    vtot *= dxdy * (double)h->Nx * (double)h->Nys;
-    std::vector<double> p;
-    cudaError_t e;
-    e = h->cfg.precision == MR_F64 ? launch_moments<double>(h->g64, (const double*)T, 0.0, 0, h->buf.red, h->red_blocks, st)
-                                   : launch_moments<float>(h->g32, (const float*)T, 0.0, 0, h->buf.red, h->red_blocks, st);
+    const double zz[2] = {h->zc[0] - h->zf[0], h->zf[h->Nz] - h->zc[h->Nz - 1]};
+    // everything is launched before the one synchronisation; the divergence depends
+    // on the velocity alone: once per velocity
+    const bool div = h->have_velocity && !h->maxdiv_valid;
+    int n = 0;
+    cudaError_t e = launch_field_moments(h, T, st);
+    if (e == cudaSuccess)
+        e = h->cfg.precision == MR_F64 ? launch_plate_nu<double>(h->g64, (const double*)T, zz, h->buf.nu2, st)
+                                       : launch_plate_nu<float>(h->g32, (const float*)T, zz, h->buf.nu2, st);
+    if (e == cudaSuccess && div) e = launch_velocity_max(h, 1, &n, st);
     if (e != cudaSuccess) return cuda_check(e, "mr_scalar_stats: launch");
-    int rc = reduce_partials(h, 2, p, st);
+    double res[8];
+    const int rc = take_results(h, true, n, res, st, "mr_scalar_stats");
     if (rc) return rc;
-    double s = 0.0, bad = 0.0;
-    for (int q = 0; q < h->red_blocks; ++q) { s += p[2 * q]; bad += p[2 * q + 1]; }
-    out->integral = s * dxdy;
-    out->mean = out->integral / vtot;
-    e = h->cfg.precision == MR_F64
-            ? launch_moments<double>(h->g64, (const double*)T, out->mean, 1, h->buf.red, h->red_blocks, st)
-            : launch_moments<float>(h->g32, (const float*)T, out->mean, 1, h->buf.red, h->red_blocks, st);
-    if (e != cudaSuccess) return cuda_check(e, "mr_scalar_stats: launch");
-    if ((rc = reduce_partials(h, 2, p, st))) return rc;
-    double v = 0.0;
-    for (int q = 0; q < h->red_blocks; ++q) v += p[2 * q];
-    out->var = v * dxdy / vtot;
-    double nu[2];
-    if ((rc = mr_plate_nu(h, nu, stream))) return rc;
-    if ((rc = cuda_check(cudaStreamSynchronize(st), "mr_scalar_stats: sync"))) return rc;
-    out->nu_bot = nu[0];
-    out->nu_top = nu[1];
-    out->max_div = 0.0;
-    if (h->have_velocity) {
-        // the divergence depends on the velocity alone: once per velocity
-        if (!h->maxdiv_valid) {
-            if ((rc = max_divergence(h, &h->maxdiv, st))) return rc;
-            h->maxdiv_valid = true;
-        }
-        out->max_div = h->maxdiv;
+    const double dxdy = (h->cfg.lx / h->Nx) * (h->cfg.ly / h->Ny), v = column_volume(h);
+    out->integral = res[0] * dxdy;
+    out->mean = res[0] / v;
+    out->var = res[1] / v;
+    out->nu_bot = res[3];
+    out->nu_top = res[4];
+    if (div) {
+        h->maxdiv = res[5];
+        h->maxdiv_valid = true;
     }
-    if (bad > 0.0) return set_error(MR_ERR_NONFINITE, "mr_scalar_stats: the scalar holds NaN or Inf");
+    out->max_div = h->have_velocity ? h->maxdiv : 0.0;
+    if (res[2] > 0.0) return set_error(MR_ERR_NONFINITE, "mr_scalar_stats: the scalar holds NaN or Inf");
     return MR_OK;
 }
 
@@ -1246,46 +1262,14 @@ int mr_cfl_dt(mr_handle h, double cfl, double* dt_out, mr_stream stream)
     if (!(cfl > 0)) return set_error(MR_ERR_ARG, "mr_cfl_dt: cfl must be positive");
     if (!h->have_velocity) return set_error(MR_ERR_STATE, "mr_cfl_dt: call mr_refine_velocity first");
     cudaStream_t st = (cudaStream_t)stream;
-    DeviceBuffers& b = h->buf;
-    const void *us = b.Us, *vs = b.Vs, *ws = b.Ws;
-    bool tmp = false;
-    cudaError_t e = cudaSuccess;
-    if (h->cfg.velocity_mode == MR_VEL_XFUSED) {
-        // the split-x kernel forms the dense faces in registers: one pass, no dense storage
-        e = launch_xfused_max_f32(h->g32, 2, b.xwy, b.xuo, b.xvr, b.nxg, b.xlc, b.xlcw, b.xrx, b.red, h->red_blocks, st);
-    } else if (h->cfg.velocity_mode == MR_VEL_FUSED) {
-        // the fused kernel forms the dense faces in registers from the coarse ones
-        e = launch_fused_max_f32(h->g32, 2, FusedInputs{b.cpad, {}, {}, 0, b.fsc, b.xlc, b.xrx, b.xry, nullptr, nullptr}, b.red,
-                                 h->red_blocks, st);
-    } else if (h->cfg.velocity_mode != MR_VEL_STORED) {
-        // dense faces are not kept: refine into temporary buffers once
-        void *a = nullptr, *bb = nullptr, *c = nullptr;
-        e = dev_malloc(&a, h->nU * h->elt);
-        if (e == cudaSuccess) e = dev_malloc(&bb, h->nV * h->elt);
-        if (e == cudaSuccess) e = dev_malloc(&c, h->nW * h->elt);
-        if (e != cudaSuccess) {
-            dev_free(a); dev_free(bb); dev_free(c);
-            return cuda_check(e, "mr_cfl_dt: temporary dense faces");
-        }
-        int rc = refine_into(h, a, bb, c, st);
-        if (rc) { dev_free(a); dev_free(bb); dev_free(c); return rc; }
-        us = a; vs = bb; ws = c;
-        tmp = true;
-    }
-    if (h->cfg.velocity_mode == MR_VEL_STORED || tmp)
-        e = h->cfg.precision == MR_F64
-                ? launch_cfl<double>(h->g64, (const double*)us, (const double*)vs, (const double*)ws, b.red, h->red_blocks, st)
-                : launch_cfl<float>(h->g32, (const float*)us, (const float*)vs, (const float*)ws, b.red, h->red_blocks, st);
-    std::vector<double> p;
-    int rc = e != cudaSuccess ? cuda_check(e, "mr_cfl_dt: launch") : reduce_partials(h, 1, p, st);
-    if (tmp) { dev_free((void*)us); dev_free((void*)vs); dev_free((void*)ws); }
+    int n = 0;
+    const cudaError_t e = launch_velocity_max(h, 2, &n, st);
+    if (e != cudaSuccess) return cuda_check(e, "mr_cfl_dt: launch");
+    double res[8];
+    const int rc = take_results(h, false, n, res, st, "mr_cfl_dt");
     if (rc) return rc;
-    if (h->cfg.velocity_mode != MR_VEL_STORED && fused_take_error(st) == MR_ERR_TIMEOUT)
-        return set_error(MR_ERR_TIMEOUT, "mr_cfl_dt: a fused kernel gave up a bounded wait");
-    double m = 0.0;
-    for (double v : p) m = std::max(m, v);
-    if (!(m > 0)) return set_error(MR_ERR_ARG, "mr_cfl_dt: zero velocity");
-    *dt_out = cfl / m;
+    if (!(res[5] > 0)) return set_error(MR_ERR_ARG, "mr_cfl_dt: zero velocity");
+    *dt_out = cfl / res[5];
     return MR_OK;
 }
 
@@ -1297,7 +1281,7 @@ int mr_debug_index_maps(mr_handle h, int32_t* out, size_t cap)
     if (cap < need) return set_error(MR_ERR_ARG, "mr_debug_index_maps: buffer too small");
     // the maps are read back from the device copy the kernels use
     std::vector<int> win(3 * ((size_t)c.nx + c.ny + c.nz));
-    const char* base = (const char*)h->buf.metric + metric_bytes<double>(h) + metric_bytes<float>(h);
+    const char* base = (const char*)h->buf.metric + metric_bytes<double>(h) + metric_bytes<float>(h) + (size_t)h->Nz * sizeof(double);
     cudaError_t e = cudaMemcpy(win.data(), base, win.size() * sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_check(e, "mr_debug_index_maps");
     int32_t* p = out;
@@ -1316,27 +1300,18 @@ namespace {
 
 using namespace mr;
 
-// FP64 volume mean and variance of a dense field in precision P (two-pass).
+// FP64 volume mean and variance of a dense field in precision P.
 int field_moments(mr_handle h, const void* T, double* mean, double* var, cudaStream_t st)
 {
-    const double dxdy = (h->cfg.lx / h->Nx) * (h->cfg.ly / h->Ny);
-    double vtot = 0.0;
-    for (int k = 0; k < h->Nz; ++k) vtot += h->dz[k];
-    vtot *= dxdy * (double)h->Nx * (double)h->Nys;
-    std::vector<double> p;
-    for (int pass = 0; pass < 2; ++pass) {
-        cudaError_t e = h->cfg.precision == MR_F64
-                            ? launch_moments<double>(h->g64, (const double*)T, *mean, pass, h->buf.red, h->red_blocks, st)
-                            : launch_moments<float>(h->g32, (const float*)T, *mean, pass, h->buf.red, h->red_blocks, st);
-        if (e != cudaSuccess) return cuda_check(e, "moments");
-        int rc = reduce_partials(h, 2, p, st);
-        if (rc) return rc;
-        double s = 0.0;
-        for (int q = 0; q < h->red_blocks; ++q) s += p[2 * q];
-        if (pass == 0) *mean = s * dxdy / vtot;
-        else *var = s * dxdy / vtot;
-    }
-    return MR_OK;
+    double res[3];
+    cudaError_t e = launch_field_moments(h, T, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(res, h->buf.mom + 1 + 6 * (size_t)kMomentBlocks, sizeof res, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const double v = column_volume(h);
+    *mean = res[0] / v;
+    *var = res[1] / v;
+    return cuda_check(e, "moments");
 }
 
 int field_nu(mr_handle h, const void* T, double nu[2], cudaStream_t st)
@@ -1563,15 +1538,14 @@ int mr_upscale_scalar(mr_handle h, double* Tc, mr_stream stream)
     cudaStream_t st = (cudaStream_t)stream;
     DeviceBuffers& b = h->buf;
     const size_t nc = (size_t)h->cfg.nx * h->nys * h->cfg.nz;
-    const size_t need = nc + (size_t)h->Nz + 1 + (size_t)h->Nz;
-    if (!b.diag) {
-        cudaError_t e = dev_malloc((void**)&b.diag, need * sizeof(double));
+    const bool dev = is_device_pointer(Tc);
+    if (!dev && !b.diag) {
+        cudaError_t e = dev_malloc((void**)&b.diag, nc * sizeof(double));
         if (e != cudaSuccess) return cuda_check(e, "mr_upscale_scalar: buffer");
     }
-    const bool dev = is_device_pointer(Tc);
     double* out = dev ? Tc : b.diag;
-    cudaError_t e = h->cfg.precision == MR_F64 ? launch_upscale<double>(h->g64, (const double*)b.T[h->ic], out, st)
-                                               : launch_upscale<float>(h->g32, (const float*)b.T[h->ic], out, st);
+    cudaError_t e = h->cfg.precision == MR_F64 ? launch_upscale<double>(h->g64, (const double*)b.T[h->ic], b.upw, out, st)
+                                               : launch_upscale<float>(h->g32, (const float*)b.T[h->ic], b.upw, out, st);
     if (e != cudaSuccess) return cuda_check(e, "mr_upscale_scalar: launch");
     if (!dev) e = cudaMemcpyAsync(Tc, out, nc * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1585,49 +1559,53 @@ int mr_scalar_profiles(mr_handle h, double* nu_z, double* nu_T, mr_stream stream
         return set_error(MR_ERR_STATE, "mr_scalar_profiles: call mr_refine_velocity and mr_set_scalar first");
     cudaStream_t st = (cudaStream_t)stream;
     DeviceBuffers& b = h->buf;
-    const size_t nc = (size_t)h->cfg.nx * h->nys * h->cfg.nz;
     if (h->slab) return set_error(MR_ERR_ARG, "mr_scalar_profiles: not on a y-slab handle");
-    if (!b.diag) {
-        cudaError_t e = dev_malloc((void**)&b.diag, (nc + 2 * (size_t)h->Nz + 1) * sizeof(double));
-        if (e != cudaSuccess) return cuda_check(e, "mr_scalar_profiles: buffer");
+    const size_t plane = (size_t)h->Nx * h->Ny;
+    cudaError_t e = cudaSuccess;
+    if (!b.prof) e = dev_malloc((void**)&b.prof, profile_work(plane, h->Nz) * sizeof(double));
+    const bool stored = h->cfg.velocity_mode == MR_VEL_STORED;
+    if (e == cudaSuccess && !stored && !b.scrW)
+        e = dev_malloc(&b.scrW, (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx * h->elt);
+    if (e != cudaSuccess) return cuda_check(e, "mr_scalar_profiles: work");
+    if (h->cfg.precision == MR_F64) {
+        e = launch_profiles<double>(h->g64, (const double*)b.T[h->ic], (const double*)b.Ws, nullptr, nullptr, nullptr, nullptr,
+                                    b.prof, st);
+    } else if (stored) {
+        e = launch_profiles<float>(h->g32, (const float*)b.T[h->ic], (const float*)b.Ws, nullptr, nullptr, nullptr, nullptr,
+                                   b.prof, st);
+    } else {
+        // the fused modes keep no dense W: the slab balance at coarse resolution here,
+        // its split in x and y in the kernel
+        e = launch_column_balance<float>(h->g32, (const float*)b.Uc, (const float*)b.Vc, (const float*)b.Wc, (float*)b.scrW, st);
+        if (e == cudaSuccess)
+            e = launch_profiles<float>(h->g32, (const float*)b.T[h->ic], nullptr, (const float*)b.Wc, (const float*)b.scrW,
+                                       b.xrx, b.xry, b.prof, st);
     }
-    double* dnu = b.diag + nc;
-    double* dzc = dnu + h->Nz + 1;
-    cudaError_t e = cudaMemcpyAsync(dzc, h->zc.data(), h->Nz * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return cuda_check(e, "mr_scalar_profiles: centres");
-    // dense W of the refinement: stored, or refined into a temporary for the fused modes
-    const void* ws = b.Ws;
-    void *tu = nullptr, *tv = nullptr, *tw = nullptr;
-    if (h->cfg.velocity_mode != MR_VEL_STORED) {
-        e = dev_malloc(&tu, h->nU * h->elt);
-        if (e == cudaSuccess) e = dev_malloc(&tv, h->nV * h->elt);
-        if (e == cudaSuccess) e = dev_malloc(&tw, h->nW * h->elt);
-        int rc = e != cudaSuccess ? cuda_check(e, "mr_scalar_profiles: temporary faces") : refine_into(h, tu, tv, tw, st);
-        if (rc) { dev_free(tu); dev_free(tv); dev_free(tw); return rc; }
-        ws = tw;
+    std::vector<double> p(8 * ((size_t)h->Nz + 1));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p.data(), b.prof, p.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_check(e, "mr_scalar_profiles");
+    const double dx = h->cfg.lx / h->Nx, dy = h->cfg.ly / h->Ny;
+    double s = 0.0, vt = 0.0;
+    for (int k = 0; k <= h->Nz; ++k) {
+        const double* q = &p[8 * (size_t)k];
+        const bool plate = k == 0 || k == h->Nz;
+        const double d = k == 0 ? h->zc[0] - h->zf[0] : (k == h->Nz ? h->zf[k] - h->zc[k - 1] : h->zc[k] - h->zc[k - 1]);
+        if (nu_z) {
+            double wt = 0.0;
+            if (!plate && h->cfg.face_order == 4)
+                for (int c = 0; c < 4; ++c) wt += h->f4z[4 * (size_t)k + c] * q[c];
+            else if (!plate)
+                wt = (h->dz[k] * q[1] + h->dz[k - 1] * q[2]) / (h->dz[k - 1] + h->dz[k]);
+            nu_z[k] = (wt / h->kappa - q[4] / d) / (double)plane;
+        }
+        if (!plate || h->cfg.bc_plates == MR_DIRICHLET) s += q[5] * dx * dy / d;
+        if (k < h->Nz) {
+            s += (q[6] * dy / dx + q[7] * dx / dy) * h->dz[k];
+            vt += h->dz[k];
+        }
     }
-    const double zb = h->zc[0] - h->zf[0], zt = h->zf[h->Nz] - h->zc[h->Nz - 1];
-    e = h->cfg.precision == MR_F64
-            ? launch_nu_profile<double>(h->g64, (const double*)b.T[h->ic], (const double*)ws, dzc, 1.0 / h->kappa, zb, zt,
-                                        dnu, b.red, h->red_blocks, st)
-            : launch_nu_profile<float>(h->g32, (const float*)b.T[h->ic], (const float*)ws, dzc, 1.0 / h->kappa, zb, zt,
-                                       dnu, b.red, h->red_blocks, st);
-    std::vector<double> p;
-    int rc = e != cudaSuccess ? cuda_check(e, "mr_scalar_profiles: launch") : reduce_partials(h, 1, p, st);
-    if (tu) { dev_free(tu); dev_free(tv); dev_free(tw); }
-    if (rc) return rc;
-    if (nu_T) {
-        double s = 0.0, vt = 0.0;
-        for (int q = 0; q < h->red_blocks; ++q) s += p[q];
-        for (int k = 0; k < h->Nz; ++k) vt += h->dz[k];
-        vt *= h->cfg.lx * h->cfg.ly;
-        *nu_T = s / vt;
-    }
-    if (nu_z) {
-        e = cudaMemcpy(nu_z, dnu, (h->Nz + 1) * sizeof(double), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_check(e, "mr_scalar_profiles: copy");
-        for (int k = 0; k <= h->Nz; ++k) nu_z[k] /= (double)h->Nx * (double)h->Ny;
-    }
+    if (nu_T) *nu_T = s / (vt * h->cfg.lx * h->cfg.ly);
     return MR_OK;
 }
 

@@ -1469,14 +1469,16 @@ int* fused_error_flag()
     return *slot;
 }
 
+int* fused_error_peek()
+{
+    std::lock_guard<std::mutex> lock(g_err_mu);
+    int** slot = err_slot();
+    return slot ? *slot : nullptr;
+}
+
 int fused_take_error(cudaStream_t st)
 {
-    int* flag = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(g_err_mu);
-        int** slot = err_slot();
-        if (slot) flag = *slot;
-    }
+    int* flag = fused_error_peek();
     if (!flag) return 0;
     int v = 0;
     if (cudaMemcpyAsync(&v, flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return MR_ERR_CUDA;

@@ -13,6 +13,7 @@
 namespace mr {
 
 constexpr int kPlateBlocks = 304;  // blocks of the plate Nusselt reduction
+constexpr int kMomentBlocks = 152 * 8;   // blocks of the volume moments
 
 // Device view of the grid and of the per-layer coefficients, in precision P.
 // Built once per handle from the FP64 host grid (Sections 3.1, 3.2).
@@ -73,6 +74,9 @@ struct DeviceBuffers {
     void* scrV = nullptr;                      // refinement scratch: full-coarse-width V per dense row
     void* metric = nullptr;                    // one block holding every Grid array
     double* red = nullptr;                     // reduction partials
+    double* mom = nullptr;                     // work of the volume moments, then 8 results (launch_gather)
+    double* prof = nullptr;                    // work of the profiles (lazy)
+    const double* upw = nullptr;               // [Nz] dz_k / (mx my sum of the slab's dz), in metric
     double* nu2 = nullptr;                     // plate Nusselt numbers (2 doubles + partials)
     void* stage = nullptr;                     // conversion staging buffer
     void* tri = nullptr;                       // implicit-z work of tall columns (zsolve_needs_work)
@@ -91,7 +95,7 @@ struct DeviceBuffers {
     double* nup = nullptr;                     // MR_VEL_FUSED: work of the plate-Nu launch (lazy)
     float xw4[8] = {0};                        // fourth order: twice the x and y face weights (uniform)
     int xlcw = 12;                             // row length of xlc
-    double* diag = nullptr;                    // diagnostics: coarse T, Nu(z), dense z centres (lazy)
+    double* diag = nullptr;                    // coarse T for a host result (lazy)
     int nxg = 0;
     // Temporal refinement (Section 3.4): the velocity of the next coarse time
     // level, in the same layout as the current one above (allocated by the
@@ -195,9 +199,21 @@ bool zsolve_needs_work(int Nz);   // whether launch_zsolve uses work (one value 
 template <typename P>
 cudaError_t launch_convert(const void* src, int src_dtype, void* dst, int dst_dtype, size_t n,
                            cudaStream_t st);
+// Sum of T dz, of (T - mean)^2 dz and the count of non-finite values into out[0..2],
+// mean being out[0] / vtot; work: 1 + 6 kMomentBlocks doubles, the first one zero
+// before the first launch (each launch leaves it zero).
 template <typename P>
-cudaError_t launch_moments(const Grid<P>& g, const P* T, double mean, int pass, double* partials,
-                           int blocks, cudaStream_t st);
+cudaError_t launch_moments(const Grid<P>& g, const P* T, const double* dz, double vtot, double* work, double* out, cudaStream_t st);
+// Sums of the heat-flux profiles, per z-face eight (mr_diag.cu: kSums), into
+// work[0 .. 8 (Nz + 1)); work: profile_work() doubles.  Ws: dense W, or NULL and W is
+// split in x and y from the full-area one of the coarse columns (Wc on the coarse
+// planes, Win on the others) with the uniform R rows rx12, ry12.
+size_t profile_work(size_t plane, int Nz);
+template <typename P>
+cudaError_t launch_profiles(const Grid<P>& g, const P* T, const P* Ws, const float* Wc, const float* Win,
+                            const float* rx12, const float* ry12, double* work, cudaStream_t st);
+// res[3..4] = nu2, res[5] = maximum of part[0..n), res[6] = *err (then cleared); each may be NULL
+cudaError_t launch_gather(const double* nu2, const double* part, int n, int* err, double* res, cudaStream_t st);
 template <typename P>
 cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* out2,
                             cudaStream_t st);
@@ -205,10 +221,7 @@ template <typename P>
 cudaError_t launch_maxdiv(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, double* partials,
                           int blocks, cudaStream_t st);
 template <typename P>
-cudaError_t launch_upscale(const Grid<P>& g, const P* T, double* Tc, cudaStream_t st);
-template <typename P>
-cudaError_t launch_nu_profile(const Grid<P>& g, const P* T, const P* Ws, const double* zc, double inv_kappa, double zb,
-                              double zt, double* nu_z, double* partials, int blocks, cudaStream_t st);
+cudaError_t launch_upscale(const Grid<P>& g, const P* T, const double* upw, double* Tc, cudaStream_t st);
 template <typename P>
 cudaError_t launch_cfl(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, double* partials,
                        int blocks, cudaStream_t st);
@@ -291,6 +304,7 @@ cudaError_t launch_adj_direct(const Grid<P>& g, const P* T, double s_nu_bottom, 
 template <typename P>
 cudaError_t launch_times_volume(const Grid<P>& g, const P* mu, int dst_dtype, void* out, cudaStream_t st);
 int fused_take_error(cudaStream_t st);   // MR_ERR_TIMEOUT if a fused kernel gave up a wait
+int* fused_error_peek();                 // the device's error flag, or NULL before any fused launch
 // Test hook (mr_debug_inject_wait_timeout): if armed, hand the next TMA step
 // launch its stop ring and wait limit, and disarm; else leave both unchanged.
 void take_wait_injection(int* stop_ring, unsigned long long* wait_ns);

@@ -1,7 +1,8 @@
-// FP64 reductions (Section 4.1 plate Nusselt numbers, volume moments, the
-// divergence check of Section 3.2, the CFL limit) and dtype conversion.
-// Each block reduces with warp shuffles into one FP64 partial; the host sums
-// the partials in block order, so every result is deterministic.
+// FP64 reductions (Section 4.1 plate Nusselt numbers, the divergence check of
+// Section 3.2, the CFL limit), the upscale integration and dtype conversion
+// (volume moments and profiles: mr_diag.cu).  Each block reduces with warp
+// shuffles into one FP64 partial, and the partials are combined in a fixed order,
+// so every result is deterministic.
 #include <math.h>
 
 #include "mr_internal.cuh"
@@ -40,64 +41,6 @@ __device__ void block_reduce_store(double (&v)[NV], double* out)
             if (lane == 0) out[q] = r;
         }
     }
-}
-
-// pass 0: (sum T vol, count of non-finite T); pass 1: sum (T - mean)^2 vol.
-// vol is dx dy dz_k; the dx dy factor is applied on the host.  Work units are
-// slices of one dense plane (8 per plane), so dz_k is common to a unit; a
-// thread loads 16 cells at a time (16 independent loads in flight), adds them
-// in precision P and each group into its FP64 sum, which is scaled by dz_k
-// once per unit.
-template <typename P>
-__global__ void __launch_bounds__(kRedThreads) k_moments(Grid<P> g, const P* __restrict__ T, double mean,
-                                                         int pass, double* __restrict__ partials)
-{
-    constexpr int kSlices = 8, kGroup = 16;
-    const size_t plane = (size_t)g.Nx * g.Ny, per = (plane + kSlices - 1) / kSlices;
-    const int units = g.Nz * kSlices;
-    const P mp = (P)mean;
-    double v[2] = {0.0, 0.0};
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
-        const int k = u / kSlices, sl = u - k * kSlices;
-        const P* r = T + (size_t)k * plane;
-        const size_t lo = (size_t)sl * per, hi = lo + per < plane ? lo + per : plane;
-        const size_t step = blockDim.x;
-        double acc = 0.0;
-        int bad = 0;
-        size_t m = lo + threadIdx.x;
-        for (; m + (kGroup - 1) * step < hi; m += kGroup * step) {
-            P t[kGroup];
-#pragma unroll
-            for (int q = 0; q < kGroup; ++q) t[q] = r[m + q * step];
-            P grp = 0;
-#pragma unroll
-            for (int q = 0; q < kGroup; ++q) {
-                if (pass == 0) {
-                    if (isfinite(t[q])) grp += t[q];
-                    else ++bad;
-                } else {
-                    const P d = t[q] - mp;
-                    grp += d * d;
-                }
-            }
-            acc += (double)grp;
-        }
-        P grp = 0;
-        for (; m < hi; m += step) {
-            const P t = r[m];
-            if (pass == 0) {
-                if (isfinite(t)) grp += t;
-                else ++bad;
-            } else {
-                const P d = t - mp;
-                grp += d * d;
-            }
-        }
-        acc += (double)grp;
-        v[0] += acc * (double)g.dz[k];
-        v[1] += (double)bad;
-    }
-    block_reduce_store<2, false>(v, partials + 2 * blockIdx.x);
 }
 
 // Plate Nusselt numbers: every block sums a fixed slice of both plates,
@@ -221,93 +164,44 @@ __global__ void __launch_bounds__(kRedThreads) k_cfl(Grid<P> g, const P* __restr
     block_reduce_store<1, true>(v, partials + blockIdx.x);
 }
 
-// Upscale integration (Section 3.3): volume average over every coarse cell.
-template <typename P>
-__global__ void k_upscale(Grid<P> g, const P* __restrict__ T, double* __restrict__ Tc)
+// VEC contiguous values as one load (1, 2 or 4 of them; aligned to their size).
+template <typename P, int VEC>
+struct alignas(sizeof(P) * VEC) Pack {
+    P v[VEC];
+};
+
+// Upscale integration (Section 3.3): volume average over every coarse cell, the
+// sum over each dense layer in the working precision (GB300's FP64 pipe is 1/64
+// of its FP32 rate), weighted in FP64 by upw[k] = dz_k / (mx my sum of the slab's
+// dz): two FP64 operations per cell and layer.  A thread owns a coarse cell and
+// reads its rows VEC values at a time.  FP32, 64 x 64 x 48 coarse cells at M = 4:
+// 10.4 us; 19.5 us with scalar loads, the weights' sum and a division per cell.
+template <typename P, int VEC, int M>
+__global__ void __launch_bounds__(128) k_upscale(Grid<P> g, const P* __restrict__ T, const double* __restrict__ upw,
+                                                 double* __restrict__ Tc)
 {
     const size_t n = (size_t)g.nz * g.ny * g.nx;
+    const int mx = M ? M : g.mx, my = M ? M : g.my, mz = M ? M : g.mz;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
         const int I = (int)(t % g.nx), J = (int)((t / g.nx) % g.ny), K = (int)(t / ((size_t)g.nx * g.ny));
-        // the sum over each dense layer in the working precision (GB300's FP64
-        // pipe is 1/64 of its FP32 rate), the volume weighting in FP64
-        double s = 0.0, h = 0.0;
-        for (int k = K * g.mz; k < (K + 1) * g.mz; ++k) {
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < mz; ++c) {
+            const int k = K * mz + c;
             P r = P(0);
-            for (int j = J * g.my; j < (J + 1) * g.my; ++j) {
-                const P* row = T + ((size_t)k * g.Ny + j) * g.Nx + (size_t)I * g.mx;
-                for (int i = 0; i < g.mx; ++i) r += row[i];
-            }
-            s += (double)r * (double)g.dz[k];
-            h += (double)g.dz[k];
-        }
-        Tc[t] = s / (h * g.mx * g.my);
-    }
-}
-
-// Nu(z) (Section 4.1) on dense z-face k = blockIdx.x: plane average of
-// w T_f / kappa - dT/dz (the plates: conductive flux only).
-template <typename P>
-__global__ void __launch_bounds__(256) k_nu_profile(Grid<P> g, const P* __restrict__ T, const P* __restrict__ Ws,
-                                                    const double* __restrict__ zc, double inv_kappa, double zb,
-                                                    double zt, double* __restrict__ nu_z)
-{
-    const int k = blockIdx.x;
-    const size_t plane = (size_t)g.Nx * g.Ny;
-    double v[1] = {0.0};
-    for (size_t m = threadIdx.x; m < plane; m += blockDim.x) {
-        if (k == 0) {
-            v[0] += (0.5 - (double)T[m]) / zb;
-        } else if (k == g.Nz) {
-            v[0] += ((double)T[(size_t)(g.Nz - 1) * plane + m] + 0.5) / zt;
-        } else {
-            const double tl = (double)T[(size_t)(k - 1) * plane + m], tr = (double)T[(size_t)k * plane + m];
-            double tf = (double)g.wlo[k] * tl + (double)g.whi[k] * tr;
-            if (g.order4) {                      // the step's fourth-order face value
-                tf = 0.0;
-                for (int q = 0; q < 4; ++q) {
-                    const int c = k - 2 + q;
-                    if (c >= 0 && c < g.Nz) tf += (double)g.f4z[4 * k + q] * (double)T[(size_t)c * plane + m];
+            const P* row = T + ((size_t)k * g.Ny + (size_t)J * my) * g.Nx + (size_t)I * mx;
+#pragma unroll
+            for (int j = 0; j < my; ++j)
+#pragma unroll
+                for (int i = 0; i < mx; i += VEC) {
+                    const Pack<P, VEC> q = *reinterpret_cast<const Pack<P, VEC>*>(row + (size_t)j * g.Nx + i);
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) r += q.v[e];
                 }
-            }
-            v[0] += (double)Ws[(size_t)k * plane + m] * tf * inv_kappa - (tr - tl) / (zc[k] - zc[k - 1]);
+            s = fma((double)r, upw[k], s);
         }
+        Tc[t] = s;
     }
-    block_reduce_store<1, false>(v, nu_z + k);
-}
-
-// <|grad T|^2> from face gradients weighted by the face's dual volume (A d),
-// plates at their Dirichlet values: partial sums per block.
-template <typename P>
-__global__ void __launch_bounds__(kRedThreads) k_grad2(Grid<P> g, const P* __restrict__ T, const double* __restrict__ zc,
-                                                       double zb, double zt, double* __restrict__ partials)
-{
-    const size_t plane = (size_t)g.Nx * g.Ny, n = plane * g.Nz;
-    const double dx = (double)g.dx, dy = (double)g.dy;
-    double v[1] = {0.0};
-    for (size_t m = (size_t)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(m % g.Nx), j = (int)((m / g.Nx) % g.Ny), k = (int)(m / plane);
-        const double t = (double)T[m], dzk = (double)g.dz[k];
-        if (!(g.walls && i == 0)) {
-            const double d = t - (double)T[m - i + (i == 0 ? g.Nx - 1 : i - 1)];
-            v[0] += d * d * dy * dzk / dx;
-        }
-        if (!(g.walls && j == 0)) {
-            const double d = t - (double)T[m + ((ptrdiff_t)(j == 0 ? g.Ny - 1 : j - 1) - j) * g.Nx];
-            v[0] += d * d * dx * dzk / dy;
-        }
-        if (k > 0) {
-            const double d = t - (double)T[m - plane];
-            v[0] += d * d * dx * dy / (zc[k] - zc[k - 1]);
-        } else if (g.dirichlet) {
-            const double d = t - 0.5;
-            v[0] += d * d * dx * dy / zb;
-        }
-        if (k == g.Nz - 1 && g.dirichlet) {
-            const double d = -0.5 - t;
-            v[0] += d * d * dx * dy / zt;
-        }
-    }
-    block_reduce_store<1, false>(v, partials + blockIdx.x);
 }
 
 template <typename S, typename D>
@@ -320,14 +214,6 @@ __global__ void k_convert(const S* __restrict__ src, D* __restrict__ dst, size_t
 }  // namespace
 
 template <typename P>
-cudaError_t launch_moments(const Grid<P>& g, const P* T, double mean, int pass, double* partials, int blocks,
-                           cudaStream_t st)
-{
-    k_moments<P><<<blocks, kRedThreads, 0, st>>>(g, T, mean, pass, partials);
-    return cudaGetLastError();
-}
-
-template <typename P>
 cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* out2, cudaStream_t st)
 {
     // out2 holds 3 + 2 * kPlateBlocks doubles: the two means, the block count
@@ -338,18 +224,17 @@ cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, d
 }
 
 template <typename P>
-cudaError_t launch_upscale(const Grid<P>& g, const P* T, double* Tc, cudaStream_t st)
+cudaError_t launch_upscale(const Grid<P>& g, const P* T, const double* upw, double* Tc, cudaStream_t st)
 {
-    k_upscale<P><<<152 * 8, kRedThreads, 0, st>>>(g, T, Tc);
-    return cudaGetLastError();
-}
-
-template <typename P>
-cudaError_t launch_nu_profile(const Grid<P>& g, const P* T, const P* Ws, const double* zc, double inv_kappa, double zb,
-                              double zt, double* nu_z, double* partials, int blocks, cudaStream_t st)
-{
-    k_nu_profile<P><<<g.Nz + 1, 256, 0, st>>>(g, T, Ws, zc, inv_kappa, zb, zt, nu_z);
-    k_grad2<P><<<blocks, kRedThreads, 0, st>>>(g, T, zc, zb, zt, partials);
+    const size_t n = (size_t)g.nz * g.ny * g.nx, want = (n + 127) / 128;
+    const unsigned blocks = (unsigned)(want < 152 * 16 ? want : 152 * 16);
+    const bool cube = g.mx == g.my && g.my == g.mz;       // unrolled: every load of a cell in flight
+    // rows of a coarse cell start at multiples of mx: whole packs where mx allows
+    // (16 bytes at most; the scalar's buffers are 256-byte aligned)
+    if (cube && g.mx == 4) k_upscale<P, sizeof(P) == 4 ? 4 : 2, 4><<<blocks, 128, 0, st>>>(g, T, upw, Tc);
+    else if (cube && g.mx == 2) k_upscale<P, 2, 2><<<blocks, 128, 0, st>>>(g, T, upw, Tc);
+    else if (g.mx % 2 == 0) k_upscale<P, 2, 0><<<blocks, 128, 0, st>>>(g, T, upw, Tc);
+    else k_upscale<P, 1, 0><<<blocks, 128, 0, st>>>(g, T, upw, Tc);
     return cudaGetLastError();
 }
 
@@ -389,14 +274,11 @@ cudaError_t launch_convert(const void* src, int sd, void* dst, int dd, size_t n,
 }
 
 #define MR_INST(P)                                                                                           \
-    template cudaError_t launch_moments<P>(const Grid<P>&, const P*, double, int, double*, int, cudaStream_t); \
     template cudaError_t launch_plate_nu<P>(const Grid<P>&, const P*, const double*, double*, cudaStream_t);    \
     template cudaError_t launch_maxdiv<P>(const Grid<P>&, const P*, const P*, const P*, double*, int,          \
                                           cudaStream_t);                                                     \
     template cudaError_t launch_cfl<P>(const Grid<P>&, const P*, const P*, const P*, double*, int, cudaStream_t);    \
-    template cudaError_t launch_upscale<P>(const Grid<P>&, const P*, double*, cudaStream_t);                       \
-    template cudaError_t launch_nu_profile<P>(const Grid<P>&, const P*, const P*, const double*, double, double,   \
-                                              double, double*, double*, int, cudaStream_t);
+    template cudaError_t launch_upscale<P>(const Grid<P>&, const P*, const double*, double*, cudaStream_t);
 MR_INST(double)
 MR_INST(float)
 #undef MR_INST
