@@ -384,7 +384,7 @@ void mr_destroy(mr_handle h)
     cudaSetDevice(h->device);
     cudaDeviceSynchronize();
     DeviceBuffers& b = h->buf;
-    void* ptrs[] = {b.T[0], b.T[1], b.T[2], b.U64, b.V64, b.W64, b.Us, b.Vs, b.Ws, b.vmax, b.scrW, b.scrV,
+    void* ptrs[] = {b.T[0], b.T[1], b.T[2], b.U64, b.V64, b.W64, b.Us, b.Vs, b.Ws, b.vmax, b.rwork, b.scrW, b.scrV,
                     b.metric, b.red, b.mom, b.prof, b.nu2, b.stage, b.tri};
     for (void* p : ptrs)
         if (p) dev_free(p);
@@ -497,8 +497,6 @@ int mr_create(const mr_config* cfg, mr_handle* out)
         alloc(&b.Vs, h->nV * h->elt);
         alloc(&b.Ws, h->nW * h->elt);
         if (h->elt == 8) alloc((void**)&b.vmax, 4 * sizeof(unsigned));
-        alloc(&b.scrW, (size_t)(h->Nz + 1) * c.ny * c.nx * h->elt);
-        alloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * c.nx * h->elt);
     }
     const size_t mb64 = metric_bytes<double>(h), mb32 = metric_bytes<float>(h);
     const size_t nwin = 3 * ((size_t)c.nx + c.ny + c.nz);
@@ -641,20 +639,27 @@ static int copy_out(mr_handle h, const void* src, int sd, void* dst, int dd, siz
     return MR_OK;
 }
 
-// Refine the handle's coarse faces into device dense-face buffers (Section 3.2).
-static int refine_into(mr_handle h, void* dUs, void* dVs, void* dWs, cudaStream_t st)
+// Refine the handle's coarse faces into device dense faces (Section 3.2); FP64:
+// with a second copy of them where given, and their largest magnitudes (vmax).
+static int refine_into(mr_handle h, void* const dense[3], void* const copy[3], unsigned* vmax, cudaStream_t st)
 {
     DeviceBuffers& b = h->buf;
     cudaError_t e = cudaSuccess;
-    if (!b.scrW) e = dev_malloc(&b.scrW, (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx * h->elt);
-    if (e == cudaSuccess && !b.scrV) e = dev_malloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * h->cfg.nx * h->elt);
-    if (e != cudaSuccess) return cuda_check(e, "refinement scratch");
-    if (h->cfg.precision == MR_F64)
-        e = launch_refine<double>(h->g64, (const double*)b.Uc, (const double*)b.Vc, (const double*)b.Wc,
-                                  (double*)dUs, (double*)dVs, (double*)dWs, (double*)b.scrW, (double*)b.scrV, st);
-    else
-        e = launch_refine<float>(h->g32, (const float*)b.Uc, (const float*)b.Vc, (const float*)b.Wc,
-                                 (float*)dUs, (float*)dVs, (float*)dWs, (float*)b.scrW, (float*)b.scrV, st);
+    if (h->cfg.precision == MR_F64) {
+        if (!b.rwork) e = dev_malloc(&b.rwork, refine_work(h->g64));
+        if (e != cudaSuccess) return cuda_check(e, "refinement work");
+        double* const d[3] = {(double*)dense[0], (double*)dense[1], (double*)dense[2]};
+        double* const c[3] = {copy ? (double*)copy[0] : nullptr, copy ? (double*)copy[1] : nullptr,
+                              copy ? (double*)copy[2] : nullptr};
+        e = launch_refine<double>(h->g64, b.U64, b.V64, b.W64, d, c, vmax, (double*)b.rwork, st);
+    } else {
+        if (!b.scrW) e = dev_malloc(&b.scrW, (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx * h->elt);
+        if (e == cudaSuccess && !b.scrV) e = dev_malloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * h->cfg.nx * h->elt);
+        if (e != cudaSuccess) return cuda_check(e, "refinement work");
+        e = launch_refine_in_place<float>(h->g32, (const float*)b.Uc, (const float*)b.Vc, (const float*)b.Wc,
+                                          (float*)dense[0], (float*)dense[1], (float*)dense[2], (float*)b.scrW,
+                                          (float*)b.scrV, st);
+    }
     return cuda_check(e, "refinement launch");
 }
 
@@ -663,9 +668,10 @@ static int refine_into(mr_handle h, void* dUs, void* dVs, void* dWs, cudaStream_
 // Load a coarse velocity into the handle's current level: FP64 copy, the
 // precision-P coarse faces, and what the velocity mode steps from (dense faces
 // for MR_VEL_STORED, the split-x intermediates for MR_VEL_XFUSED).
-static int derive_velocity(mr_handle h, bool convert, cudaStream_t st);
+static int derive_velocity(mr_handle h, bool convert, cudaStream_t st, void* const copy[3] = nullptr);
 
-static int load_velocity(mr_handle h, const double* U, const double* V, const double* W, cudaStream_t st)
+static int load_velocity(mr_handle h, const double* U, const double* V, const double* W, cudaStream_t st,
+                         void* const copy[3] = nullptr)
 {
     DeviceBuffers& b = h->buf;
     int rc;
@@ -687,12 +693,13 @@ static int load_velocity(mr_handle h, const double* U, const double* V, const do
         if ((rc = copy_in(h, V, MR_F64, b.V64, MR_F64, h->ncV, st))) return rc;
         if ((rc = copy_in(h, W, MR_F64, b.W64, MR_F64, h->ncW, st))) return rc;
     }
-    return derive_velocity(h, !fetched, st);
+    return derive_velocity(h, !fetched, st, copy);
 }
 
 // What the velocity mode steps from, given the FP64 coarse faces in U64/V64/W64
-// (and, unless convert, their FP32 rounding already in Uc/Vc/Wc).
-static int derive_velocity(mr_handle h, bool convert, cudaStream_t st)
+// (and, unless convert, their FP32 rounding already in Uc/Vc/Wc).  copy: where
+// MR_VEL_STORED writes the dense faces a second time (device memory), or NULL.
+static int derive_velocity(mr_handle h, bool convert, cudaStream_t st, void* const copy[3])
 {
     DeviceBuffers& b = h->buf;
     h->maxdiv_valid = false;
@@ -720,10 +727,8 @@ static int derive_velocity(mr_handle h, bool convert, cudaStream_t st)
         if (e != cudaSuccess) return cuda_check(e, "padded coarse faces");
     }
     if (h->cfg.velocity_mode == MR_VEL_STORED) {
-        const int rc = refine_into(h, b.Us, b.Vs, b.Ws, st);
-        if (rc || !b.vmax) return rc;
-        return cuda_check(launch_vmax((const double*)b.Us, h->nU, (const double*)b.Vs, h->nV, (const double*)b.Ws,
-                                      h->nW, b.vmax, st), "velocity maxima");
+        void* const dense[3] = {b.Us, b.Vs, b.Ws};
+        return refine_into(h, dense, copy, b.vmax, st);
     }
     return MR_OK;
 }
@@ -887,12 +892,16 @@ int mr_refine_velocity(mr_handle h, const double* U, const double* V, const doub
     if (Us && h->slab) return set_error(MR_ERR_ARG, "mr_refine_velocity: no dense faces from a y-slab handle");
     cudaStream_t st = (cudaStream_t)stream;
     DeviceBuffers& b = h->buf;
-    int rc = load_velocity(h, U, V, W, st);
+    // FP64 dense faces given out in device memory are written with the handle's own
+    void* const copy[3] = {Us, Vs, Ws};
+    const bool stored = h->cfg.velocity_mode == MR_VEL_STORED;
+    const bool direct = Us && stored && h->elt == 8 && is_device_pointer(Us) && is_device_pointer(Vs) && is_device_pointer(Ws);
+    int rc = load_velocity(h, U, V, W, st, direct ? copy : nullptr);
     if (rc) return rc;
     h->have_velocity = true;
-    if (!Us) return MR_OK;
+    if (!Us || direct) return MR_OK;
     const int P = h->cfg.precision;
-    if (h->cfg.velocity_mode != MR_VEL_STORED) return refine_into(h, Us, Vs, Ws, st);
+    if (!stored) return refine_into(h, copy, nullptr, nullptr, st);
     if ((rc = copy_out(h, b.Us, P, Us, P, h->nU, st))) return rc;
     if ((rc = copy_out(h, b.Vs, P, Vs, P, h->nV, st))) return rc;
     return copy_out(h, b.Ws, P, Ws, P, h->nW, st);

@@ -70,8 +70,9 @@ struct DeviceBuffers {
     void* Vs = nullptr;
     void* Ws = nullptr;
     unsigned* vmax = nullptr;                  // MR_VEL_STORED, FP64: largest |U|, |V|, |W| (high words)
-    void* scrW = nullptr;                      // refinement scratch: full-coarse-area W per dense plane
-    void* scrV = nullptr;                      // refinement scratch: full-coarse-width V per dense row
+    void* rwork = nullptr;                     // FP64: work of the dense refinement (refine_work)
+    void* scrW = nullptr;                      // FP32: full-coarse-area W per dense plane
+    void* scrV = nullptr;                      // FP32: full-coarse-width V per dense row
     void* metric = nullptr;                    // one block holding every Grid array
     double* red = nullptr;                     // reduction partials
     double* mom = nullptr;                     // work of the volume moments, then 8 results (launch_gather)
@@ -172,9 +173,18 @@ bool is_device_pointer(const void* p);
 StepCoef step_coef(const mr_config& cfg, int64_t s);
 
 // launchers (return cudaError_t of the launch)
+// FP64: the dense faces out[3] (and, unless NULL, a second copy of them in copy[3]);
+// vmax (may be NULL): the largest magnitudes of the components; work: refine_work bytes.
 template <typename P>
-cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* Us, P* Vs, P* Ws,
-                          P* scrW, P* scrV, cudaStream_t st);
+size_t refine_work(const Grid<P>& g);
+template <typename P>
+cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* const out[3], P* const copy[3],
+                          unsigned* vmax, P* work, cudaStream_t st);
+// The same with little more memory than the outputs (slower): scrW (Nz + 1) ny nx,
+// scrV Nz (Ny + w) nx values.
+template <typename P>
+cudaError_t launch_refine_in_place(const Grid<P>& g, const P* U, const P* V, const P* W, P* Us, P* Vs, P* Ws, P* scrW,
+                                   P* scrV, cudaStream_t st);
 template <typename P>
 cudaError_t launch_step_stored(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, const P* Tm1,
                                const P* T, P* Tp1, StepCoef c, bool implz, cudaStream_t st);
@@ -184,8 +194,6 @@ bool step_fix_fits(const Grid<double>& g);
 cudaError_t launch_step_fix(const Grid<double>& g, const double* Us, const double* Vs, const double* Ws,
                             const double* Tm1, const double* T, double* Tp1, StepCoef c, bool implz,
                             const unsigned* vmax, cudaStream_t st);
-cudaError_t launch_vmax(const double* U, size_t nU, const double* V, size_t nV, const double* W, size_t nW,
-                        unsigned* vmax, cudaStream_t st);
 // the same step with the velocity A + alpha (B - A) of two stored dense fields
 template <typename P>
 cudaError_t launch_step_stored_lerp(const Grid<P>& g, const P* const velA[3], const P* const velB[3], double alpha,

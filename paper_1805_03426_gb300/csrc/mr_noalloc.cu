@@ -209,6 +209,6 @@ extern "C" int mr_refine_velocity_noalloc(const mr_config* c, const double* U, c
     g.dz = (const double*)(b + oDz);
     g.Rx = (const double*)(b + oRx); g.Ry = (const double*)(b + oRy); g.Rz = (const double*)(b + oRz);
     g.wx = wx; g.wy = wx + 3 * c->nx; g.wz = wx + 3 * (c->nx + c->ny);
-    e = launch_refine<double>(g, U, V, W, Us, Vs, Ws, (double*)(b + oSW), (double*)(b + oSV), st);
+    e = launch_refine_in_place<double>(g, U, V, W, Us, Vs, Ws, (double*)(b + oSW), (double*)(b + oSV), st);
     return cuda_check(e, "mr_refine_velocity_noalloc: refinement launch");
 }

@@ -380,23 +380,6 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
     }
 }
 
-// Largest magnitude (the high word of |v|) of each face component into vmax[0..2].
-__global__ void __launch_bounds__(256) k_vmax(const double* __restrict__ U, size_t nU, const double* __restrict__ V,
-                                              size_t nV, const double* __restrict__ W, size_t nW,
-                                              unsigned* __restrict__ vmax)
-{
-    const double* p[3] = {U, V, W};
-    const size_t n[3] = {nU, nV, nW};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        unsigned m = 0;
-        for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n[c]; q += (size_t)gridDim.x * blockDim.x)
-            m = max(m, mag(p[c][q]));
-        m = __reduce_max_sync(0xffffffffu, m);
-        if ((threadIdx.x & 31) == 0 && m) atomicMax(vmax + c, m);
-    }
-}
-
 template <int R>
 cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
 {
@@ -427,15 +410,6 @@ cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
 }
 
 }  // namespace
-
-cudaError_t launch_vmax(const double* U, size_t nU, const double* V, size_t nV, const double* W, size_t nW,
-                        unsigned* vmax, cudaStream_t st)
-{
-    cudaError_t e = cudaMemsetAsync(vmax, 0, 3 * sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-    k_vmax<<<152 * 8, 256, 0, st>>>(U, nU, V, nV, W, nW, vmax);
-    return cudaGetLastError();
-}
 
 // Grids it takes: 32-bit byte offsets inside a plane, second-order faces, and at
 // least 196,608 cells.  Below that too few warps march too long a chain, and one
