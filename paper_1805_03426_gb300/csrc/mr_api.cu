@@ -665,10 +665,10 @@ static int refine_into(mr_handle h, void* const dense[3], void* const copy[3], u
 
 }  // extern "C"
 
-// Load a coarse velocity into the handle's current level: FP64 copy, the
-// precision-P coarse faces, and what the velocity mode steps from (dense faces
+// Load a coarse velocity into the handle's current level: the coarse faces in the
+// handle's precision, and what the velocity mode steps from (dense faces
 // for MR_VEL_STORED, the split-x intermediates for MR_VEL_XFUSED).
-static int derive_velocity(mr_handle h, bool convert, cudaStream_t st, void* const copy[3] = nullptr);
+static int derive_velocity(mr_handle h, const double* const src[3], cudaStream_t st, void* const copy[3] = nullptr);
 
 static int load_velocity(mr_handle h, const double* U, const double* V, const double* W, cudaStream_t st,
                          void* const copy[3] = nullptr)
@@ -676,7 +676,12 @@ static int load_velocity(mr_handle h, const double* U, const double* V, const do
     DeviceBuffers& b = h->buf;
     int rc;
     const bool f32 = h->cfg.precision == MR_F32;
-    bool fetched = false;
+    if (f32 && is_device_pointer(U) && is_device_pointer(V) && is_device_pointer(W)) {
+        // device faces of an FP32 handle: converted from where they are, no FP64 copy
+        const double* const src[3] = {U, V, W};
+        return derive_velocity(h, src, st);
+    }
+    const double* const own[3] = {b.U64, b.V64, b.W64};
     const double *mU = host_mapped(U), *mV = host_mapped(V), *mW = host_mapped(W);
     if (mU && mV && mW) {
         // pinned host faces: the SMs read them over the host link, writing the
@@ -684,36 +689,34 @@ static int load_velocity(mr_handle h, const double* U, const double* V, const do
         cudaError_t e = launch_fetch_f64(mU, b.U64, f32 ? (float*)b.Uc : nullptr, h->ncU, st);
         if (e == cudaSuccess) e = launch_fetch_f64(mV, b.V64, f32 ? (float*)b.Vc : nullptr, h->ncV, st);
         if (e == cudaSuccess) e = launch_fetch_f64(mW, b.W64, f32 ? (float*)b.Wc : nullptr, h->ncW, st);
-        if (e == cudaErrorInvalidValue) cudaGetLastError();   // unaligned: the copy path below
-        else if (e != cudaSuccess) return cuda_check(e, "fetch coarse faces");
-        else fetched = true;
+        if (e == cudaSuccess) return derive_velocity(h, nullptr, st, copy);
+        if (e != cudaErrorInvalidValue) return cuda_check(e, "fetch coarse faces");
+        cudaGetLastError();                               // unaligned: the copy path below
     }
-    if (!fetched) {
-        if ((rc = copy_in(h, U, MR_F64, b.U64, MR_F64, h->ncU, st))) return rc;
-        if ((rc = copy_in(h, V, MR_F64, b.V64, MR_F64, h->ncV, st))) return rc;
-        if ((rc = copy_in(h, W, MR_F64, b.W64, MR_F64, h->ncW, st))) return rc;
-    }
-    return derive_velocity(h, !fetched, st, copy);
+    if ((rc = copy_in(h, U, MR_F64, b.U64, MR_F64, h->ncU, st))) return rc;
+    if ((rc = copy_in(h, V, MR_F64, b.V64, MR_F64, h->ncV, st))) return rc;
+    if ((rc = copy_in(h, W, MR_F64, b.W64, MR_F64, h->ncW, st))) return rc;
+    return derive_velocity(h, own, st, copy);
 }
 
-// What the velocity mode steps from, given the FP64 coarse faces in U64/V64/W64
-// (and, unless convert, their FP32 rounding already in Uc/Vc/Wc).  copy: where
-// MR_VEL_STORED writes the dense faces a second time (device memory), or NULL.
-static int derive_velocity(mr_handle h, bool convert, cudaStream_t st, void* const copy[3])
+// What the velocity mode steps from, given the FP64 coarse faces src in device
+// memory (FP64 handles: U64/V64/W64), or, src NULL, their FP32 rounding already in
+// Uc/Vc/Wc.  copy: where MR_VEL_STORED writes the dense faces a second time (FP64,
+// device memory), or NULL.
+static int derive_velocity(mr_handle h, const double* const src[3], cudaStream_t st, void* const copy[3])
 {
     DeviceBuffers& b = h->buf;
     h->maxdiv_valid = false;
-    if (h->cfg.velocity_mode == MR_VEL_FUSED && convert) {
+    if (h->cfg.velocity_mode == MR_VEL_FUSED && src) {
         // the FP64 faces straight to the padded FP32 copy (and the FP32 faces)
-        cudaError_t e = launch_fused_pad64(b.U64, b.V64, b.W64, b.cpad, (float*)b.Uc, (float*)b.Vc, (float*)b.Wc,
+        cudaError_t e = launch_fused_pad64(src[0], src[1], src[2], b.cpad, (float*)b.Uc, (float*)b.Vc, (float*)b.Wc,
                                            h->cfg.nx, h->cfg.ny, h->cfg.nz, h->slab ? h->cfg.slab_j0 : 0, h->nys, st);
         return cuda_check(e, "padded coarse faces");
     }
-    if (h->cfg.precision == MR_F32 && convert) {
-        // the handle's own FP64 device faces: no pointer queries
-        cudaError_t e = launch_convert<double>(b.U64, MR_F64, b.Uc, MR_F32, h->ncU, st);
-        if (e == cudaSuccess) e = launch_convert<double>(b.V64, MR_F64, b.Vc, MR_F32, h->ncV, st);
-        if (e == cudaSuccess) e = launch_convert<double>(b.W64, MR_F64, b.Wc, MR_F32, h->ncW, st);
+    if (h->cfg.precision == MR_F32 && src) {
+        cudaError_t e = launch_convert<double>(src[0], MR_F64, b.Uc, MR_F32, h->ncU, st);
+        if (e == cudaSuccess) e = launch_convert<double>(src[1], MR_F64, b.Vc, MR_F32, h->ncV, st);
+        if (e == cudaSuccess) e = launch_convert<double>(src[2], MR_F64, b.Wc, MR_F32, h->ncW, st);
         if (e != cudaSuccess) return cuda_check(e, "coarse faces to FP32");
     }
     if (h->cfg.velocity_mode == MR_VEL_XFUSED) {
@@ -971,7 +974,8 @@ int mr_refine_velocity_staged(mr_handle h, mr_stream stream)
         b.Wc = b.W64;
     }
     b.stg_ready = -1;
-    int rc = derive_velocity(h, true, st);
+    const double* const own[3] = {b.U64, b.V64, b.W64};
+    int rc = derive_velocity(h, own, st);
     e = cudaEventRecord(b.stg_free[q], st);
     if (rc) return rc;
     if (e != cudaSuccess) return cuda_check(e, "mr_refine_velocity_staged: record");
@@ -1005,6 +1009,9 @@ int mr_scalar_coarse_step(mr_handle h, const double* U, const double* V, const d
     return MR_OK;
 }
 
+// The level before the current one: before the first step the scalar itself.
+static const void* previous_level(mr_handle h) { return h->buf.T[h->step == 0 ? h->ic : h->ip]; }
+
 int mr_set_scalar(mr_handle h, const void* T0, int32_t dtype, mr_stream stream)
 {
     if (!h || !T0) return set_error(MR_ERR_ARG, "mr_set_scalar: NULL argument");
@@ -1012,10 +1019,8 @@ int mr_set_scalar(mr_handle h, const void* T0, int32_t dtype, mr_stream stream)
     cudaStream_t st = (cudaStream_t)stream;
     h->ip = 0;
     h->ic = 1;
+    // T^{-1} is T^0 (previous_level): one level is written, not two
     int rc = copy_in(h, T0, dtype, h->buf.T[h->ic], h->cfg.precision, h->ncell, st);
-    if (rc) return rc;
-    rc = cuda_check(cudaMemcpyAsync(h->buf.T[h->ip], h->buf.T[h->ic], h->ncell * h->elt,
-                                    cudaMemcpyDeviceToDevice, st), "mr_set_scalar");
     if (rc) return rc;
     h->step = 0;
     h->have_scalar = true;
@@ -1033,7 +1038,7 @@ int mr_get_scalar(mr_handle h, void* T, void* Tprev, int32_t dtype, mr_stream st
     if (h->cfg.velocity_mode != MR_VEL_STORED && fused_take_error(st) == MR_ERR_TIMEOUT)
         return set_error(MR_ERR_TIMEOUT, "mr_get_scalar: a fused step kernel gave up a bounded wait");
     if (T && (rc = copy_out(h, h->buf.T[h->ic], h->cfg.precision, T, dtype, h->ncell, st))) return rc;
-    if (Tprev && (rc = copy_out(h, h->buf.T[h->ip], h->cfg.precision, Tprev, dtype, h->ncell, st))) return rc;
+    if (Tprev && (rc = copy_out(h, previous_level(h), h->cfg.precision, Tprev, dtype, h->ncell, st))) return rc;
     return MR_OK;
 }
 
@@ -1408,7 +1413,7 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
         const void* Tc = h->buf.T[h->ic];
         if (s < nsteps && s % ck == 0) {
             char* pair = (char*)a.cp + (size_t)(s / ck) * 2 * fb;
-            e = cudaMemcpyAsync(pair, h->buf.T[h->ip], fb, cudaMemcpyDeviceToDevice, st);
+            e = cudaMemcpyAsync(pair, previous_level(h), fb, cudaMemcpyDeviceToDevice, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(pair + fb, Tc, fb, cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: checkpoint");
         }

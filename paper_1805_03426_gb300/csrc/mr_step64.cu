@@ -119,6 +119,8 @@ __device__ __forceinline__ long long zflux(Bal tb, Bal tt, Bal wlo, Bal whi, Bal
 template <int R, bool WALLS, bool LF>
 __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
 {
+    after_previous();
+    let_next();
     const Grid<double>& g = A.g;
     __shared__ LayerK sk[kMaxChunk];
     __shared__ Bal sc[4];                                 // 4 S_U hx, 4 S_V hy, kx2, ky2
@@ -405,8 +407,7 @@ cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
         }
     }
     const dim3 grd((unsigned)blocks, (unsigned)((g.Nz + A.kc - 1) / A.kc));
-    k<<<grd, 32 * kWarps, smem, st>>>(A);
-    return cudaGetLastError();
+    return launch_after(k, grd, 32 * kWarps, smem, st, A);
 }
 
 }  // namespace

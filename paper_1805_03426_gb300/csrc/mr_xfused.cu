@@ -180,6 +180,10 @@ k_xfused(const __grid_constant__ XMaps T, const XArgs A)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    if constexpr (KIND == 0) {
+        after_previous();
+        let_next();
+    }
 
     // ---------------------------------------------------------------- producer warp
     if (warp == NW) {
@@ -885,6 +889,7 @@ cudaError_t launch_xt(const Grid<float>& g, XSet v0, XSet v1, float alpha, int n
         memcpy(A.w4y, w4 + 4, sizeof A.w4y);
     }
     dim3 grid(chunks, g.Nx / kTX, g.Ny / TY);
+    if (KIND == 0) return launch_after(k_xfused<M, KIND, LF, MT, O4, TY>, grid, L::THREADS, L::bytes, st, maps, A);
     k_xfused<M, KIND, LF, MT, O4, TY><<<grid, L::THREADS, L::bytes, st>>>(maps, A);
     return cudaGetLastError();
 }

@@ -8,6 +8,7 @@ fallback: if ``libmr.so`` is missing, importing the binding fails loudly.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 
 import numpy as np
@@ -105,45 +106,55 @@ def _check(rc):
         raise MRError(rc, lib().mr_last_error().decode())
 
 
+_torch = None       # the torch module once it has been found, False without it
+
+
+def _find_torch():
+    global _torch
+    if _torch is None:
+        try:
+            import torch
+            _torch = torch
+        except ImportError:  # pragma: no cover
+            _torch = False
+    return _torch
+
+
 def _ptr(a, n=None, dtype=None, what="array"):
     """Raw pointer of a contiguous torch tensor or numpy array (None -> NULL)."""
     if a is None:
         return None
-    try:
-        import torch
-        is_t = isinstance(a, torch.Tensor)
-    except ImportError:  # pragma: no cover
-        is_t = False
-    if is_t:
+    torch = _torch or _find_torch()
+    if torch and isinstance(a, torch.Tensor):
         if not a.is_contiguous():
             raise ValueError(f"{what}: tensor must be contiguous")
-        size, dt = a.numel(), {a.dtype}
-        ok = {np.float64: "torch.float64", np.float32: "torch.float32"}
-        if dtype is not None and str(a.dtype) != ok[dtype]:
-            raise TypeError(f"{what}: expected {ok[dtype]}, got {a.dtype}")
+        size = a.numel()
+        if dtype is not None and a.dtype != (torch.float64 if dtype is np.float64 else torch.float32):
+            raise TypeError(f"{what}: expected torch.{np.dtype(dtype).name}, got {a.dtype}")
         p = a.data_ptr()
     else:
         if not isinstance(a, np.ndarray) or not a.flags["C_CONTIGUOUS"]:
             raise ValueError(f"{what}: numpy array must be C-contiguous")
         if dtype is not None and a.dtype != dtype:
             raise TypeError(f"{what}: expected {np.dtype(dtype)}, got {a.dtype}")
-        size, dt = a.size, None
+        size = a.size
         p = a.ctypes.data
-    del dt
     if n is not None and size != n:
         raise ValueError(f"{what}: {size} elements, expected {n}")
     return p
 
 
+_cuda = False       # whether torch has found a GPU
+
+
 def _stream(stream):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
-    try:
-        import torch
-        if torch.cuda.is_available():
-            return torch.cuda.current_stream().cuda_stream
-    except ImportError:  # pragma: no cover
-        pass
+    global _cuda
+    torch = _torch or _find_torch()
+    if torch and (_cuda or torch.cuda.is_available()):
+        _cuda = True
+        return torch.cuda.current_stream().cuda_stream
     return None
 
 
@@ -198,7 +209,7 @@ class Handle:
 
 
 def _n(shape):
-    return int(np.prod(shape))
+    return math.prod(shape)
 
 
 def mr_create(cfg: mr_config) -> Handle:
