@@ -56,6 +56,8 @@ __global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P,
                                                      const P* __restrict__ Tm1, const P* __restrict__ T,
                                                      P* __restrict__ Tp1, P a, P b, P gdt)
 {
+    after_previous();
+    let_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
@@ -138,6 +140,8 @@ __global__ void __launch_bounds__(256) k_step_periodic(Grid<P> g, const P* __res
                                                        const P* __restrict__ Tm1, const P* __restrict__ T,
                                                        P* __restrict__ Tp1, P a, P b, P gdt)
 {
+    after_previous();
+    let_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
@@ -161,6 +165,74 @@ __global__ void __launch_bounds__(256) k_step_periodic(Grid<P> g, const P* __res
     const P D = L[7] + g.kx2 * (Tm1[mw] + Tm1[me]) + g.ky2 * (Tm1[ms] + Tm1[mn]) + L[4] * Db + L[5] * Dt + L[6] * Dc;
     const P C = g.hx * ax + g.hy * ay + az;
     Tp1[m] = LF ? Dc + gdt * (C + D) : a * Dc + b * Tc + gdt * (C + D);
+}
+
+// The FP32 form of k_step_periodic on rows of whole quads: a thread marches four
+// cells of a row through kMarch layers, so that its loads are 16 bytes wide and the
+// planes above become the current ones and those below in registers.  The
+// operations are k_step_periodic's in its order and with its contractions (spelt
+// out here), so that the results are the same to the last bit: the FP32 adjoint's
+// coarse gradients magnify any other rounding of the forward run by 1e4.
+// Bound by L2 and the loads' latency on grids that fit L2: 128 x 128 x 96 cells
+// 7.6 us per step, 14.8 us with a cell per thread (back to back); 512 x 512 x 384:
+// 467 and 870 us.
+constexpr int kMarch = 4;
+__device__ __forceinline__ float get(const float4& v, int q) { return q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w)); }
+__device__ __forceinline__ void put(float4& v, int q, float x) { (q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w))) = x; }
+template <bool LF>
+__global__ void __launch_bounds__(128) k_step_periodic4(Grid<float> g, const float* __restrict__ Us,
+                                                        const float* __restrict__ Vs, const float* __restrict__ Ws,
+                                                        const float* __restrict__ Tm1, const float* __restrict__ T,
+                                                        float* __restrict__ Tp1, float a, float b, float gdt, int march)
+{
+    after_previous();
+    let_next();
+    const unsigned quads = (unsigned)g.Nx / 4, s = blockIdx.x * 128u + threadIdx.x;
+    if (s >= quads * (unsigned)g.Ny) return;
+    const int j = (int)(s / quads), i = (int)(s % quads) * 4;
+    const int k0 = blockIdx.y * march, k1 = min(k0 + march, g.Nz);
+    const size_t plane = (size_t)g.Nx * g.Ny, row = (size_t)j * g.Nx + i;
+    const size_t west = row - i + (i == 0 ? g.Nx - 1 : i - 1), east = row - i + (i + 4 == g.Nx ? 0 : i + 4);
+    const size_t south = (size_t)(j == 0 ? g.Ny - 1 : j - 1) * g.Nx + i, north = (size_t)(j == g.Ny - 1 ? 0 : j + 1) * g.Nx + i;
+    auto quad = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    size_t m = (size_t)k0 * plane;
+    float4 tb = k0 > 0 ? quad(T + m - plane + row) : zero, db = k0 > 0 ? quad(Tm1 + m - plane + row) : zero;
+    float4 tc = quad(T + m + row), dc = quad(Tm1 + m + row), wb = quad(Ws + m + row);
+    for (int k = k0; k < k1; ++k, m += plane) {
+        const float* L = g.lz + 8 * k;
+        const bool hi = k < g.Nz - 1;
+        const float4 tt = hi ? quad(T + m + plane + row) : zero, dt = hi ? quad(Tm1 + m + plane + row) : zero;
+        const float4 wt = quad(Ws + m + plane + row);
+        const float4 ts = quad(T + m + south), tn = quad(T + m + north), ds = quad(Tm1 + m + south), dn = quad(Tm1 + m + north);
+        const float4 u = quad(Us + m + row), vs = quad(Vs + m + row), vn = quad(Vs + m + north);
+        const float tw = T[m + west], te = T[m + east], dw = Tm1[m + west], de = Tm1[m + east], ue = Us[m + east];
+        float4 out;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float Tc = get(tc, q), Dc = get(dc, q);
+            const float Tw = q ? get(tc, q - 1) : tw, Te = q < 3 ? get(tc, q + 1) : te;
+            const float Dw = q ? get(dc, q - 1) : dw, De = q < 3 ? get(dc, q + 1) : de;
+            const float U0 = get(u, q), U1 = q < 3 ? get(u, q + 1) : ue;
+            const float ax = __fmaf_rn(U0, __fadd_rn(Tw, Tc), -__fmul_rn(U1, __fadd_rn(Tc, Te)));
+            const float ay = __fmaf_rn(get(vs, q), __fadd_rn(get(ts, q), Tc), -__fmul_rn(get(vn, q), __fadd_rn(Tc, get(tn, q))));
+            const float az = __fmaf_rn(get(wb, q), __fmaf_rn(L[0], get(tb, q), __fmul_rn(L[1], Tc)),
+                                       __fmul_rn(get(wt, q), __fmaf_rn(L[2], Tc, __fmul_rn(L[3], get(tt, q)))));
+            float D = __fmaf_rn(g.kx2, __fadd_rn(Dw, De), L[7]);
+            D = __fmaf_rn(g.ky2, __fadd_rn(get(ds, q), get(dn, q)), D);
+            D = __fmaf_rn(L[4], get(db, q), D);
+            D = __fmaf_rn(L[5], get(dt, q), D);
+            D = __fmaf_rn(L[6], Dc, D);
+            const float C = __fadd_rn(__fmaf_rn(g.hx, ax, __fmul_rn(g.hy, ay)), az), S = __fadd_rn(C, D);
+            put(out, q, LF ? __fmaf_rn(gdt, S, Dc) : __fmaf_rn(gdt, S, __fmaf_rn(a, Dc, __fmul_rn(b, Tc))));
+        }
+        *reinterpret_cast<float4*>(Tp1 + m + row) = out;
+        tb = tc;
+        db = dc;
+        tc = tt;
+        dc = dt;
+        wb = wt;
+    }
 }
 
 // Opt-in implicit vertical diffusion: per (x, y) column solve
@@ -297,7 +369,10 @@ cudaError_t zsolve_table(const Grid<P>& g, P* X, double h, const double* cdn, co
     const size_t plane = (size_t)g.Nx * g.Ny;
     const unsigned blocks = (unsigned)((plane + 15) / 16);
     const int bytes = (g.Nz - M) * 32 * (int)sizeof(P);
-    // at least four blocks of one warp per SM (one per scheduler); beyond that y goes
+    // Launched when the step has finished: one-warp blocks that come up while it still
+    // runs gather on the SMs that empty first, several to a scheduler, whose FP64 pipe
+    // bounds them (70 instead of 57 us per step on 123 x 74 x 148 cells).
+    // At least four blocks of one warp per SM (one per scheduler); beyond that y goes
     // through global memory
     if (bytes <= 56 * 1024) {
         static unsigned long long done = 0;                // one bit per device
@@ -319,25 +394,34 @@ cudaError_t step_stored(const Grid<P>& g, const FaceVel<P, LERP>& u, const FaceV
     dim3 grd((g.Nx + blk.x - 1) / blk.x, (g.Ny + blk.y - 1) / blk.y, g.Nz);
     const P a = (P)c.a, b = (P)c.b, gdt = (P)c.gdt;
     if (!LERP && !implz && !g.order4 && !g.walls) {
-        if (c.a == 1.0 && c.b == 0.0)
-            k_step_periodic<P, true><<<grd, blk, 0, st>>>(g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
-        else
-            k_step_periodic<P, false><<<grd, blk, 0, st>>>(g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
-        return cudaGetLastError();
+        if constexpr (sizeof(P) == 4) {
+            // whole quads, 16-byte aligned
+            const uintptr_t all = reinterpret_cast<uintptr_t>(u.A) | reinterpret_cast<uintptr_t>(v.A) |
+                                  reinterpret_cast<uintptr_t>(w.A) | reinterpret_cast<uintptr_t>(Tm1) |
+                                  reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(Tp1);
+            const size_t quads = (size_t)(g.Nx / 4) * g.Ny;
+            // fewer layers per thread where the grid would not give every SM 256 threads
+            int march = kMarch;
+            while (march > 1 && quads * ((g.Nz + march - 1) / march) < 152 * 256) march /= 2;
+            const size_t layers = (g.Nz + march - 1) / march;
+            if (g.Nx % 4 == 0 && !(all & 15) && quads < (1u << 31) && layers <= 65535)
+                return launch_after(c.a == 1.0 && c.b == 0.0 ? k_step_periodic4<true> : k_step_periodic4<false>,
+                                    dim3((unsigned)((quads + 127) / 128), (unsigned)layers), 128, 0, st, g, u.A, v.A, w.A,
+                                    Tm1, T, Tp1, a, b, gdt, march);
+        }
+        return launch_after(c.a == 1.0 && c.b == 0.0 ? k_step_periodic<P, true> : k_step_periodic<P, false>, grd, blk, 0, st,
+                            g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
     }
-    if (g.order4) {
-        if (implz) k_step_stored<P, true, LERP, true><<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
-        else k_step_stored<P, false, LERP, true><<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
-    } else {
-        if (implz) k_step_stored<P, true, LERP, false><<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
-        else k_step_stored<P, false, LERP, false><<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
-    }
-    return cudaGetLastError();
+    return launch_after(g.order4 ? (implz ? k_step_stored<P, true, LERP, true> : k_step_stored<P, false, LERP, true>)
+                                 : (implz ? k_step_stored<P, true, LERP, false> : k_step_stored<P, false, LERP, false>),
+                        grd, blk, 0, st, g, u, v, w, Tm1, T, Tp1, a, b, gdt);
 }
 
 __global__ void k_lerp(const float* __restrict__ A, const float* __restrict__ B, float alpha, float* __restrict__ out,
                        size_t n)
 {
+    after_previous();
+    let_next();
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
         const float a = A[t];
         out[t] = a + alpha * (B[t] - a);
@@ -351,8 +435,7 @@ cudaError_t launch_lerp_f32(const float* A, const float* B, double alpha, float*
     if (!n) return cudaSuccess;
     const size_t want = (n + 255) / 256;
     const unsigned blocks = (unsigned)(want < 152 * 16 ? want : 152 * 16);
-    k_lerp<<<blocks, 256, 0, st>>>(A, B, (float)alpha, out, n);
-    return cudaGetLastError();
+    return launch_after(k_lerp, blocks, 256, 0, st, A, B, (float)alpha, out, n);
 }
 
 template <typename P>
