@@ -289,185 +289,215 @@ __global__ void k_times_volume(Grid<P> g, const P* __restrict__ mu, int dst_f64,
 }
 
 // ------------------------------------------------------------- refinement transpose (FP64)
-// The passes of the refinement in reverse order, each replaced by its
-// adjoint; scatter-adds use FP64 atomics.
+// The transpose of the refinement axis by axis (the stages of launch_refine in
+// mr_refine.cu in reverse order).  A balance's transpose is a running sum over the
+// faces it formed, which takes the place of their gradients; each neighbour then
+// gathers its differences.  A split's transpose sums a coarse cell's dense values
+// with the R columns first (t_p = sum_a R[a][p] x_a) and adds the three t_p to the
+// window's cells with FP64 atomics, one for each coarse value at the resolution
+// still left instead of nine products and atomics per dense face.
+//   aUs (per coarse cell in x)  -> h_a = sum_{a' >= a} aU_a'     (h_0: aUO)
+//   aVs, aWs + differences of h -> R_x^T -> aVR, aWY
+//   aVR (per coarse row)        -> g_b = sum_{b' >= b} aVR_b'    (g_0: aVZ)
+//   aUO, aWY + differences of g -> R_y^T -> aUZ, aWC
+//   aWC (per coarse slab)       -> S_c = dz_c sum_{c' <= c} aWC_c', their last sum to gW
+//   aUZ, aVZ + differences of S -> R_z^T -> gU, gV
+// 128 x 128 x 96 dense cells at M = 2: 91 us; 300 us face by face, nine atomics each.
 
-__global__ void k_t_stage_x(Grid<double> g, double* aUs, double* aVs, double* aWs)
+struct Transpose {
+    Grid<double> g;
+    double *aUs, *aVs, *aWs;         // dense face gradients (consumed)
+    double *aVR, *aWY, *aUZ, *aWC;   // zero before
+    double *gU, *gV, *gW;            // zero before
+};
+
+__device__ __forceinline__ void add(double* p, double v) { atomicAdd(p, v); }
+
+// Running sums of the x balances: thread per (layer, dense row, coarse column).
+__global__ void k_t_sum_x(const Transpose A)
 {
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)g.Nz * g.Ny * g.nx;
+    const Grid<double>& g = A.g;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, n = (size_t)g.Nz * g.Ny * g.nx;
     if (t >= n) return;
-    const int I = (int)(t % g.nx), j = (int)((t / g.nx) % g.Ny), k = (int)(t / ((size_t)g.nx * g.Ny));
-    const int jn = g.walls ? j + 1 : (j + 1) % g.Ny;
-    const double dzk = g.dz[k];
-    const size_t urow = ((size_t)k * g.Ny + j) * g.ufx;
-    double aH = 0.0;
-    for (int a = g.mx - 2; a >= 0; --a) {
-        const int i = I * g.mx + a;
-        aH += aUs[urow + i + 1] / (g.dy * dzk);
-        aUs[urow + i + 1] = 0.0;
-        atomicAdd(&aVs[((size_t)k * g.vfy + jn) * g.Nx + i], -aH * g.dx * dzk);
-        atomicAdd(&aVs[((size_t)k * g.vfy + j) * g.Nx + i], aH * g.dx * dzk);
-        atomicAdd(&aWs[((size_t)(k + 1) * g.Ny + j) * g.Nx + i], -aH * g.dx * g.dy);
-        atomicAdd(&aWs[((size_t)k * g.Ny + j) * g.Nx + i], aH * g.dx * g.dy);
+    const size_t row = t / g.nx;
+    double* u = A.aUs + row * g.ufx + (t - row * g.nx) * g.mx;
+    double h = u[g.mx - 1];
+    for (int a = g.mx - 2; a >= 0; --a) u[a] = h += u[a];
+}
+
+// R_x^T: thread per (layer, V face row, coarse column), then (plane, dense row, coarse column).
+__global__ void k_t_split_x(const Transpose A)
+{
+    const Grid<double>& g = A.g;
+    const size_t nv = (size_t)g.Nz * g.vfy * g.nx, nw = (size_t)(g.Nz + 1) * g.Ny * g.nx;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nv + nw) return;
+    const bool v = t < nv;
+    const size_t e = v ? t : t - nv, row = e / g.nx;
+    const int I = (int)(e - row * g.nx), rows = v ? g.vfy : g.Ny, k = (int)(row / rows), j = (int)(row - (size_t)k * rows);
+    // the two balances that read the face: with its coefficient in the first one
+    const double *h0 = nullptr, *h1 = nullptr;
+    double c0 = 0.0, c1 = 0.0;
+    if (v) {
+        const int js = j > 0 ? j - 1 : (g.walls ? -1 : g.Ny - 1);
+        if (j < g.Ny) h0 = A.aUs + ((size_t)k * g.Ny + j) * g.ufx;
+        if (js >= 0) h1 = A.aUs + ((size_t)k * g.Ny + js) * g.ufx;
+        c0 = c1 = g.dx / g.dy;
+    } else {
+        if (k < g.Nz) h0 = A.aUs + ((size_t)k * g.Ny + j) * g.ufx, c0 = g.dx * g.inv_dz[k];
+        if (k > 0) h1 = A.aUs + ((size_t)(k - 1) * g.Ny + j) * g.ufx, c1 = g.dx * g.inv_dz[k - 1];
     }
-    atomicAdd(&aUs[urow + (size_t)I * g.mx], aH * g.dy * dzk);
-}
-
-__global__ void k_t_split_v(Grid<double> g, double* aVs, double* aVrow)
-{
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t rows = (size_t)g.ny * (g.my - 1), n = (size_t)g.Nz * rows * g.Nx;
-    if (t >= n) return;
-    const int i = (int)(t % g.Nx), jj = (int)((t / g.Nx) % rows), k = (int)(t / ((size_t)g.Nx * rows));
-    const int j = (jj / (g.my - 1)) * g.my + jj % (g.my - 1) + 1;
-    const int I = i / g.mx;
-    const size_t f = ((size_t)k * g.vfy + j) * g.Nx + i;
-    const double v = aVs[f];
-    aVs[f] = 0.0;
-    for (int p = 0; p < 3; ++p)
-        atomicAdd(&aVrow[((size_t)k * g.vfy + j) * g.nx + g.wx[3 * I + p]], g.Rx[3 * i + p] * v);
-}
-
-__global__ void k_t_row_balance(Grid<double> g, double* aUs, double* aVs, double* aWs, const double* aVrow)
-{
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)g.Nz * g.ny * g.nx;
-    if (t >= n) return;
-    const int I = (int)(t % g.nx), J = (int)((t / g.nx) % g.ny), k = (int)(t / ((size_t)g.nx * g.ny));
-    const int Ie = g.walls ? I + 1 : (I + 1) % g.nx;
-    const double dzk = g.dz[k];
-    double aG = 0.0;
-    for (int b = g.my - 2; b >= 0; --b) {
-        const int j = J * g.my + b;
-        aG += aVrow[((size_t)k * g.vfy + j + 1) * g.nx + I] / (g.DX * dzk);
-        const size_t urow = ((size_t)k * g.Ny + j) * g.ufx;
-        atomicAdd(&aUs[urow + (size_t)Ie * g.mx], -aG * g.dy * dzk);
-        atomicAdd(&aUs[urow + (size_t)I * g.mx], aG * g.dy * dzk);
-        for (int a = 0; a < g.mx; ++a) {
-            atomicAdd(&aWs[((size_t)(k + 1) * g.Ny + j) * g.Nx + I * g.mx + a], -aG * g.dy * g.dx);
-            atomicAdd(&aWs[((size_t)k * g.Ny + j) * g.Nx + I * g.mx + a], aG * g.dy * g.dx);
+    const double* x = (v ? A.aVs : A.aWs) + row * g.Nx + (size_t)I * g.mx;
+    const double* r = g.Rx + 3 * (size_t)I * g.mx;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int a = 0; a < g.mx; ++a) {
+        double y = x[a];
+        if (a < g.mx - 1) {
+            const size_t f = (size_t)I * g.mx + a + 1;
+            if (h0) y = fma(c0, h0[f], y);
+            if (h1) y = fma(-c1, h1[f], y);
         }
+        for (int p = 0; p < 3; ++p) s[p] = fma(r[3 * a + p], y, s[p]);
     }
-    for (int a = 0; a < g.mx; ++a)
-        atomicAdd(&aVs[((size_t)k * g.vfy + (size_t)J * g.my) * g.Nx + I * g.mx + a], aG * dzk * g.dx);
+    double* o = (v ? A.aVR : A.aWY) + row * g.nx;
+    for (int p = 0; p < 3; ++p) add(o + g.wx[3 * I + p], s[p]);
 }
 
-__global__ void k_t_split_w(Grid<double> g, double* aWs, double* aWc)
+// Running sums of the row balances: thread per (layer, coarse row, coarse column).
+__global__ void k_t_sum_y(const Transpose A)
 {
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t planes = (size_t)g.nz * (g.mz - 1), n = planes * g.Ny * g.Nx;
+    const Grid<double>& g = A.g;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, n = (size_t)g.Nz * g.ny * g.nx;
     if (t >= n) return;
-    const int i = (int)(t % g.Nx), j = (int)((t / g.Nx) % g.Ny), kk = (int)(t / ((size_t)g.Nx * g.Ny));
-    const int k = (kk / (g.mz - 1)) * g.mz + kk % (g.mz - 1) + 1;
-    const int I = i / g.mx, J = j / g.my;
-    const size_t f = ((size_t)k * g.Ny + j) * g.Nx + i;
-    const double v = aWs[f];
-    aWs[f] = 0.0;
-    for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q)
-            atomicAdd(&aWc[((size_t)k * g.ny + g.wy[3 * J + q]) * g.nx + g.wx[3 * I + p]],
-                      g.Rx[3 * i + p] * g.Ry[3 * j + q] * v);
+    const size_t row = t / g.nx, k = row / g.ny;
+    double* v = A.aVR + (k * g.vfy + (row - k * g.ny) * g.my) * g.nx + (t - row * g.nx);
+    double s = v[(size_t)(g.my - 1) * g.nx];
+    for (int b = g.my - 2; b >= 0; --b) v[(size_t)b * g.nx] = s += v[(size_t)b * g.nx];
 }
 
-__global__ void k_t_column_balance(Grid<double> g, const double* aWc, double* gU, double* gV, double* gW)
+// R_y^T: thread per (layer, coarse row, U face column), then (plane, coarse row, coarse column).
+__global__ void k_t_split_y(const Transpose A)
 {
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)g.nz * g.ny * g.nx;
-    if (t >= n) return;
-    const int I = (int)(t % g.nx), J = (int)((t / g.nx) % g.ny), K = (int)(t / ((size_t)g.nx * g.ny));
-    const int Ie = g.walls ? I + 1 : (I + 1) % g.nx;
-    const int Jn = g.walls ? J + 1 : (J + 1) % g.ny;
-    double aF = 0.0;
-    for (int c = 1; c <= g.mz - 1; ++c) {
-        const int k = K * g.mz + c;
-        aF += aWc[((size_t)k * g.ny + J) * g.nx + I] / (g.DX * g.DY);
-        const double au = aF * g.DY * g.dz[k], av = aF * g.DX * g.dz[k];
-        for (int q = 0; q < 3; ++q) {
-            const double r = g.Rz[3 * k + q];
-            const int Kq = g.wz[3 * K + q];
-            atomicAdd(&gU[((size_t)Kq * g.ny + J) * g.cux + Ie], r * au);
-            atomicAdd(&gU[((size_t)Kq * g.ny + J) * g.cux + I], -r * au);
-            atomicAdd(&gV[((size_t)Kq * g.cvy + Jn) * g.nx + I], r * av);
-            atomicAdd(&gV[((size_t)Kq * g.cvy + J) * g.nx + I], -r * av);
+    const Grid<double>& g = A.g;
+    const size_t nu = (size_t)g.Nz * g.ny * g.cux, nw = (size_t)(g.Nz + 1) * g.ny * g.nx;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nu + nw) return;
+    const bool u = t < nu;
+    const int cols = u ? g.cux : g.nx;
+    const size_t e = u ? t : t - nu, row = e / cols;
+    const int I = (int)(e - row * cols), k = (int)(row / g.ny), J = (int)(row - (size_t)k * g.ny);
+    const double *g0 = nullptr, *g1 = nullptr;            // running sums of V, [dense row][coarse column]
+    double c0 = 0.0, c1 = 0.0;
+    if (u) {
+        const int Iw = I > 0 ? I - 1 : (g.walls ? -1 : g.nx - 1);
+        if (I < g.nx) g0 = A.aVR + (size_t)k * g.vfy * g.nx + I;
+        if (Iw >= 0) g1 = A.aVR + (size_t)k * g.vfy * g.nx + Iw;
+        c0 = c1 = g.dy / g.DX;
+    } else {
+        if (k < g.Nz) g0 = A.aVR + (size_t)k * g.vfy * g.nx + I, c0 = g.dy * g.inv_dz[k];
+        if (k > 0) g1 = A.aVR + (size_t)(k - 1) * g.vfy * g.nx + I, c1 = g.dy * g.inv_dz[k - 1];
+    }
+    // U's values are the running sums' first ones of each coarse cell
+    const double* x = u ? A.aUs + (size_t)k * g.Ny * g.ufx + (size_t)I * g.mx : A.aWY + (size_t)k * g.Ny * g.nx + I;
+    const size_t xs = u ? g.ufx : g.nx;
+    const double* r = g.Ry + 3 * (size_t)J * g.my;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int b = 0; b < g.my; ++b) {
+        const size_t j = (size_t)J * g.my + b;
+        double y = x[j * xs];
+        if (b < g.my - 1) {
+            if (g0) y = fma(c0, g0[(j + 1) * g.nx], y);
+            if (g1) y = fma(-c1, g1[(j + 1) * g.nx], y);
         }
+        for (int p = 0; p < 3; ++p) s[p] = fma(r[3 * b + p], y, s[p]);
     }
-    atomicAdd(&gW[((size_t)(K + 1) * g.ny + J) * g.nx + I], aF * g.DX * g.DY);
+    double* o = (u ? A.aUZ : A.aWC) + (size_t)k * g.ny * cols + I;
+    for (int p = 0; p < 3; ++p) add(o + (size_t)g.wy[3 * J + p] * cols, s[p]);
 }
 
-__global__ void k_t_outer_u(Grid<double> g, const double* aUs, double* gU)
+// Running sums of the slab balances, and W's gradient: thread per coarse cell.
+__global__ void k_t_sum_z(const Transpose A)
 {
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)g.Nz * g.Ny * g.cux;
+    const Grid<double>& g = A.g;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, plane = (size_t)g.ny * g.nx, n = (size_t)g.nz * plane;
     if (t >= n) return;
-    const int I = (int)(t % g.cux), j = (int)((t / g.cux) % g.Ny), k = (int)(t / ((size_t)g.cux * g.Ny));
-    const int J = j / g.my, K = k / g.mz;
-    const double v = aUs[((size_t)k * g.Ny + j) * g.ufx + (size_t)I * g.mx];
-    for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q)
-            atomicAdd(&gU[((size_t)g.wz[3 * K + q] * g.ny + g.wy[3 * J + p]) * g.cux + I], g.Ry[3 * j + p] * g.Rz[3 * k + q] * v);
+    const size_t K = t / plane;
+    double* w = A.aWC + K * g.mz * plane + (t - K * plane);
+    add(A.gW + t, w[0]);
+    if (K + 1 == (size_t)g.nz) add(A.gW + t + plane, w[(size_t)g.mz * plane]);
+    double s = 0.0;
+    for (int c = 1; c < g.mz; ++c) {
+        s += w[(size_t)c * plane];
+        w[(size_t)c * plane] = s * g.dz[K * g.mz + c];
+    }
+    add(A.gW + t + plane, s);
 }
 
-__global__ void k_t_outer_v(Grid<double> g, const double* aVs, double* gV)
+// R_z^T: thread per coarse U face, then per coarse V face.
+__global__ void k_t_split_z(const Transpose A)
 {
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)g.Nz * g.cvy * g.Nx;
-    if (t >= n) return;
-    const int i = (int)(t % g.Nx), J = (int)((t / g.Nx) % g.cvy), k = (int)(t / ((size_t)g.Nx * g.cvy));
-    const int I = i / g.mx, K = k / g.mz;
-    const double v = aVs[((size_t)k * g.vfy + (size_t)J * g.my) * g.Nx + i];
-    for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q)
-            atomicAdd(&gV[((size_t)g.wz[3 * K + q] * g.cvy + J) * g.nx + g.wx[3 * I + p]], g.Rx[3 * i + p] * g.Rz[3 * k + q] * v);
-}
-
-__global__ void k_t_outer_w(Grid<double> g, const double* aWs, double* gW)
-{
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t n = (size_t)(g.nz + 1) * g.Ny * g.Nx;
-    if (t >= n) return;
-    const int i = (int)(t % g.Nx), j = (int)((t / g.Nx) % g.Ny), K = (int)(t / ((size_t)g.Nx * g.Ny));
-    const int I = i / g.mx, J = j / g.my;
-    const double v = aWs[((size_t)K * g.mz * g.Ny + j) * g.Nx + i];
-    for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 3; ++q)
-            atomicAdd(&gW[((size_t)K * g.ny + g.wy[3 * J + q]) * g.nx + g.wx[3 * I + p]], g.Rx[3 * i + p] * g.Ry[3 * j + q] * v);
+    const Grid<double>& g = A.g;
+    const size_t pu = (size_t)g.ny * g.cux, pv = (size_t)g.cvy * g.nx, nu = g.nz * pu, nv = g.nz * pv;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nu + nv) return;
+    const bool u = t < nu;
+    const size_t e = u ? t : t - nu, pl = u ? pu : pv;
+    const int K = (int)(e / pl), cols = u ? g.cux : g.nx, J = (int)(e % pl / cols), I = (int)(e % pl % cols);
+    // the cells east / north (coefficient -) and west / south (+) of the face
+    const int Ie = u ? (I < g.nx ? I : -1) : I, Iw = u ? (I > 0 ? I - 1 : (g.walls ? -1 : g.nx - 1)) : I;
+    const int Jn = u ? J : (J < g.ny ? J : -1), Js = u ? J : (J > 0 ? J - 1 : (g.walls ? -1 : g.ny - 1));
+    const double c = u ? 1.0 / g.DX : 1.0 / g.DY;
+    const size_t wp = (size_t)g.ny * g.nx;
+    const double* x = u ? A.aUZ + (size_t)J * g.cux + I : A.aVR + (size_t)J * g.my * g.nx + I;
+    const size_t xs = u ? pu : (size_t)g.vfy * g.nx;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int b = 0; b < g.mz; ++b) {
+        const size_t k = (size_t)K * g.mz + b;
+        double y = x[k * xs];
+        if (b > 0) {
+            const double* S = A.aWC + k * wp;
+            double d = 0.0;
+            if (Iw >= 0 && Js >= 0) d += S[(size_t)Js * g.nx + Iw];
+            if (Ie >= 0 && Jn >= 0) d -= S[(size_t)Jn * g.nx + Ie];
+            y = fma(c, d, y);
+        }
+        for (int p = 0; p < 3; ++p) s[p] = fma(g.Rz[3 * k + p], y, s[p]);
+    }
+    double* o = (u ? A.gU : A.gV) + e % pl;
+    for (int p = 0; p < 3; ++p) add(o + (size_t)g.wz[3 * K + p] * pl, s[p]);
 }
 
 }  // namespace
 
-// P^T: dense face gradients (consumed) -> coarse gradients (zeroed first).
-cudaError_t launch_refine_transpose(const Grid<double>& g, double* aUs, double* aVs, double* aWs, double* aWc,
-                                    double* aVrow, double* gU, double* gV, double* gW, size_t ncU, size_t ncV,
-                                    size_t ncW, cudaStream_t st)
+size_t transpose_work(const Grid<double>& g)
 {
+    return (size_t)g.Nz * g.vfy * g.nx + (size_t)(g.Nz + 1) * g.ny * g.nx;
+}
+size_t transpose_wy(const Grid<double>& g) { return (size_t)(g.Nz + 1) * g.Ny * g.nx; }
+
+// P^T: dense face gradients (U, V and W one after the other; consumed) -> coarse
+// gradients (zeroed first).  The gradient of the faces refined in z alone takes the
+// place of the V and W faces, which are no longer needed by then.
+cudaError_t launch_refine_transpose(const Grid<double>& g, double* faces, double* work, double* wy, double* gU, double* gV,
+                                    double* gW, size_t ncU, size_t ncV, size_t ncW, cudaStream_t st)
+{
+    Transpose A{g, faces, nullptr, nullptr, work, wy, nullptr, nullptr, gU, gV, gW};
+    A.aVs = faces + (size_t)g.Nz * g.Ny * g.ufx;
+    A.aWs = A.aVs + (size_t)g.Nz * g.vfy * g.Nx;
+    A.aWC = work + (size_t)g.Nz * g.vfy * g.nx;
+    A.aUZ = A.aVs;
     cudaError_t e;
     if ((e = cudaMemsetAsync(gU, 0, ncU * 8, st)) || (e = cudaMemsetAsync(gV, 0, ncV * 8, st)) ||
-        (e = cudaMemsetAsync(gW, 0, ncW * 8, st)))
+        (e = cudaMemsetAsync(gW, 0, ncW * 8, st)) || (e = cudaMemsetAsync(work, 0, transpose_work(g) * 8, st)) ||
+        (e = cudaMemsetAsync(wy, 0, transpose_wy(g) * 8, st)))
         return e;
-    if ((e = cudaMemsetAsync(aWc, 0, (size_t)(g.Nz + 1) * g.ny * g.nx * 8, st)) ||
-        (e = cudaMemsetAsync(aVrow, 0, (size_t)g.Nz * g.vfy * g.nx * 8, st)))
-        return e;
-    size_t n;
-    if (g.mx > 1) { n = (size_t)g.Nz * g.Ny * g.nx; k_t_stage_x<<<nblk(n), kThreads, 0, st>>>(g, aUs, aVs, aWs); }
-    if (g.my > 1) {
-        n = (size_t)g.Nz * g.ny * (g.my - 1) * g.Nx;
-        k_t_split_v<<<nblk(n), kThreads, 0, st>>>(g, aVs, aVrow);
-        n = (size_t)g.Nz * g.ny * g.nx;
-        k_t_row_balance<<<nblk(n), kThreads, 0, st>>>(g, aUs, aVs, aWs, aVrow);
-    }
-    if (g.mz > 1) {
-        n = (size_t)g.nz * (g.mz - 1) * g.Ny * g.Nx;
-        k_t_split_w<<<nblk(n), kThreads, 0, st>>>(g, aWs, aWc);
-        n = (size_t)g.nz * g.ny * g.nx;
-        k_t_column_balance<<<nblk(n), kThreads, 0, st>>>(g, aWc, gU, gV, gW);
-    }
-    n = (size_t)g.Nz * g.Ny * g.cux;
-    k_t_outer_u<<<nblk(n), kThreads, 0, st>>>(g, aUs, gU);
-    n = (size_t)g.Nz * g.cvy * g.Nx;
-    k_t_outer_v<<<nblk(n), kThreads, 0, st>>>(g, aVs, gV);
-    n = (size_t)(g.nz + 1) * g.Ny * g.Nx;
-    k_t_outer_w<<<nblk(n), kThreads, 0, st>>>(g, aWs, gW);
+    k_t_sum_x<<<nblk((size_t)g.Nz * g.Ny * g.nx), kThreads, 0, st>>>(A);
+    k_t_split_x<<<nblk((size_t)g.Nz * g.vfy * g.nx + (size_t)(g.Nz + 1) * g.Ny * g.nx), kThreads, 0, st>>>(A);
+    if ((e = cudaMemsetAsync(A.aUZ, 0, (size_t)g.Nz * g.ny * g.cux * 8, st))) return e;
+    k_t_sum_y<<<nblk((size_t)g.Nz * g.ny * g.nx), kThreads, 0, st>>>(A);
+    k_t_split_y<<<nblk((size_t)g.Nz * g.ny * g.cux + (size_t)(g.Nz + 1) * g.ny * g.nx), kThreads, 0, st>>>(A);
+    k_t_sum_z<<<nblk((size_t)g.nz * g.ny * g.nx), kThreads, 0, st>>>(A);
+    k_t_split_z<<<nblk(g.nz * ((size_t)g.ny * g.cux + (size_t)g.cvy * g.nx)), kThreads, 0, st>>>(A);
     return cudaGetLastError();
 }
 

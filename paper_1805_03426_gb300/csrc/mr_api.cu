@@ -1384,9 +1384,9 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
     if (!a.cp) {
         e = dev_malloc(&a.cp, cpairs * 2 * fb);
         if (e == cudaSuccess) e = dev_malloc(&a.seg, ((size_t)ck + 1) * fb);
-        if (e == cudaSuccess) e = dev_malloc(&a.mu, 3 * fb);
+        if (e == cudaSuccess) e = dev_malloc(&a.mu, std::max(3 * fb, transpose_wy(h->g64) * sizeof(double)));
         if (e == cudaSuccess) e = dev_malloc((void**)&a.face, (h->nU + h->nV + h->nW) * sizeof(double));
-        const size_t nscr = (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx + (size_t)h->Nz * (h->Ny + h->w) * h->cfg.nx;
+        const size_t nscr = transpose_work(h->g64);
         if (e == cudaSuccess) e = dev_malloc((void**)&a.scr, nscr * sizeof(double));
         if (e == cudaSuccess) e = dev_malloc((void**)&a.out, (h->ncell + h->ncU + h->ncV + h->ncW) * sizeof(double));
         if (e == cudaSuccess && h->cfg.precision == MR_F32) {
@@ -1528,9 +1528,8 @@ int mr_adjoint_backward(mr_handle h, double gscale, void* gT0, int32_t gT0_dtype
         double* cU = out + h->ncell;
         double* cV = cU + h->ncU;
         double* cW = cV + h->ncV;
-        double* aWc = a.scr;
-        double* aVrow = a.scr + (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx;
-        e = launch_refine_transpose(h->g64, fU, fV, fW, aWc, aVrow, cU, cV, cW, h->ncU, h->ncV, h->ncW, st);
+        // the adjoint levels make room for the transpose's wy
+        e = launch_refine_transpose(h->g64, a.face, a.scr, (double*)a.mu, cU, cV, cW, h->ncU, h->ncV, h->ncW, st);
         if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_backward: refinement transpose");
         if (gU && (rc = copy_out(h, cU, MR_F64, gU, MR_F64, h->ncU, st))) return rc;
         if (gV && (rc = copy_out(h, cV, MR_F64, gV, MR_F64, h->ncV, st))) return rc;

@@ -185,7 +185,7 @@ struct mr_handle_s {
         void* mu = nullptr;                    // three adjoint levels
         double* face = nullptr;                // dense face gradients (U, V, W), FP64
         float* face32 = nullptr;               // MR_F32: per-segment FP32 sums, flushed into face
-        double* scr = nullptr;                 // transpose scratch (full-area W, full-width V), FP64
+        double* scr = nullptr;                 // work of the refinement's transpose, FP64
         double* out = nullptr;                 // FP64 staging of the outputs (dense T0, coarse U, V, W)
     } adj;
 };
@@ -323,9 +323,10 @@ cudaError_t launch_step_xfused_f32(const Grid<float>& g, const float* const setA
 cudaError_t launch_xfused_max_f32(const Grid<float>& g, int kind, const float* WY, const float* UO, const float* VR,
                                   int nxg, const float* lc, int lcw, const float* rx12, double* partials, int blocks,
                                   cudaStream_t st);
-cudaError_t launch_refine_transpose(const Grid<double>& g, double* aUs, double* aVs, double* aWs, double* aWc,
-                                    double* aVrow, double* gU, double* gV, double* gW, size_t ncU, size_t ncV,
-                                    size_t ncW, cudaStream_t st);
+size_t transpose_work(const Grid<double>& g);   // doubles of launch_refine_transpose's work
+size_t transpose_wy(const Grid<double>& g);     // and of its wy
+cudaError_t launch_refine_transpose(const Grid<double>& g, double* faces, double* work, double* wy, double* gU, double* gV,
+                                    double* gW, size_t ncU, size_t ncV, size_t ncW, cudaStream_t st);
 template <typename P>
 cudaError_t launch_adj_step(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, const P* T, const P* Tprev,
                             const P* Mn, P* Mc, P* Mp, double s_nu, double s_var, double mean_prev, P* gU,
