@@ -1488,7 +1488,11 @@ int mr_adjoint_backward(mr_handle h, double gscale, void* gT0, int32_t gT0_dtype
             const StepCoef co = step_coef(h->cfg, s);
             const bool euler = (s == 0);
             const int64_t sp = euler ? 0 : s - 1;
-            if (P == MR_F64)
+            if (P == MR_F64 && adj_fix_fits(h->g64))
+                e = launch_adj_fix(h->g64, (const double*)b.Us, (const double*)b.Vs, (const double*)b.Ws, (const double*)Ts,
+                                   (const double*)Tsm, (const double*)mu[in], (double*)mu[ic], (double*)mu[ip], s_nu(sp),
+                                   s_var(sp), a.mean[sp], fU, fV, fW, co, euler, b.vmax, st);
+            else if (P == MR_F64)
                 e = launch_adj_step<double>(h->g64, (const double*)b.Us, (const double*)b.Vs, (const double*)b.Ws,
                                             (const double*)Ts, (const double*)Tsm, (const double*)mu[in],
                                             (double*)mu[ic], (double*)mu[ip], s_nu(sp), s_var(sp), a.mean[sp], fU, fV,

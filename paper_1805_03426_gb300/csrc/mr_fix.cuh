@@ -76,5 +76,41 @@ __host__ __device__ __forceinline__ long long dec(int hi, int lo, int E)
     return (long long)((unsigned long long)(unsigned)((int)(r >> 32) ^ s) << 32 | (unsigned)((int)r ^ s));
 }
 
+#ifdef __CUDACC__
+__device__ __forceinline__ double pow2(int n) { return __hiloint2double((n + 1023) << 20, 0); }
+__device__ __forceinline__ Bal fixed(double v) { return bal(__double2ll_rn(v)); }
+// the magnitude of a double, ordered like its high word without the sign
+__device__ __forceinline__ unsigned mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+template <int BITS>
+__device__ __forceinline__ long long dec(double v, int E)
+{
+    return fix::dec<BITS>(__double2hiint(v), __double2loint(v), E);
+}
+
+// 2^-900 <= v < 2^900, without an FP64 comparison
+__device__ __forceinline__ bool ordinary(double v)
+{
+    return (unsigned)__double2hiint(v) - (123u << 20) < (1800u << 20);
+}
+
+// asynchronous 8-byte copies into shared memory
+__device__ __forceinline__ void copy8(double* dst, const double* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ const double* at(const double* base, unsigned bytes)
+{
+    return reinterpret_cast<const double*>(reinterpret_cast<const char*>(base) + bytes);
+}
+#endif
+
 }  // namespace fix
 }  // namespace mr

@@ -331,6 +331,12 @@ template <typename P>
 cudaError_t launch_adj_step(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, const P* T, const P* Tprev,
                             const P* Mn, P* Mc, P* Mp, double s_nu, double s_var, double mean_prev, P* gU,
                             P* gV, P* gW, StepCoef c, bool euler, cudaStream_t st);
+// the FP64 backward step with fixed-point advection and diffusion (mr_adjoint64.cu)
+bool adj_fix_fits(const Grid<double>& g);
+cudaError_t launch_adj_fix(const Grid<double>& g, const double* Us, const double* Vs, const double* Ws, const double* T,
+                           const double* Tprev, const double* Mn, double* Mc, double* Mp, double s_nu, double s_var,
+                           double mean_prev, double* gU, double* gV, double* gW, StepCoef c, bool euler,
+                           const unsigned* vmax, cudaStream_t st);
 cudaError_t launch_flush_faces(float* seg, double* tot, size_t n, cudaStream_t st);
 template <typename P>
 cudaError_t launch_adj_direct(const Grid<P>& g, const P* T, double s_nu_bottom, double s_var, double mean, P* mu,

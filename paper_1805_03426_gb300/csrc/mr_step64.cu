@@ -77,34 +77,8 @@ struct Args {
     int kc;
 };
 
-__device__ __forceinline__ double pow2(int n) { return __hiloint2double((n + 1023) << 20, 0); }
-__device__ __forceinline__ Bal fixed(double v) { return bal(__double2ll_rn(v)); }
 
-// asynchronous 8-byte copies into shared memory
-__device__ __forceinline__ void copy8(double* dst, const double* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void copy_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ const double* at(const double* base, unsigned bytes)
-{
-    return reinterpret_cast<const double*>(reinterpret_cast<const char*>(base) + bytes);
-}
 constexpr int stage_rows(int R) { return 5 * R + 5; }
-
-__device__ __forceinline__ unsigned mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
-
-template <int BITS>
-__device__ __forceinline__ long long dec(double v, int E)
-{
-    return fix::dec<BITS>(__double2hiint(v), __double2loint(v), E);
-}
 
 // z-face flux 2 T_f w from the values below and above (60-bit), their weights
 // and w (62-bit)
@@ -285,7 +259,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
                     }
                 }
             }
-            plain = !(gs > 1e-290 && gs < 1e290);
+            plain = !ordinary(gs);
         }
         if (plain) {
             // FP64 arithmetic with the same shared fluxes; the bottom faces' are
