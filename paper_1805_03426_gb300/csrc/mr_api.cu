@@ -407,7 +407,7 @@ void mr_destroy(mr_handle h)
         if (b.stg_copied[q]) cudaEventDestroy(b.stg_copied[q]);
         if (b.stg_free[q]) cudaEventDestroy(b.stg_free[q]);
     }
-    void* aptrs[] = {h->adj.cp, h->adj.seg, h->adj.mu, h->adj.face, h->adj.scr, h->adj.out};
+    void* aptrs[] = {h->adj.cp, h->adj.seg, h->adj.mu, h->adj.face, h->adj.face32, h->adj.scr, h->adj.out, h->adj.res};
     for (void* p : aptrs)
         if (p) dev_free(p);
     if (h->elt == 4) {
@@ -1129,8 +1129,8 @@ int mr_scalar_step_coupled(mr_handle h, double* nu2, double* Tc, mr_stream strea
         if (dnu) {
             const double zz[2] = {h->zc[0] - h->zf[0], h->zf[h->Nz] - h->zc[h->Nz - 1]};
             e = h->cfg.precision == MR_F64
-                    ? launch_plate_nu<double>(h->g64, (const double*)h->buf.T[h->ic], zz, h->buf.nu2, st)
-                    : launch_plate_nu<float>(h->g32, (const float*)h->buf.T[h->ic], zz, h->buf.nu2, st);
+                    ? launch_plate_nu<double>(h->g64, (const double*)h->buf.T[h->ic], zz, h->buf.nu2, h->buf.nu2, st)
+                    : launch_plate_nu<float>(h->g32, (const float*)h->buf.T[h->ic], zz, h->buf.nu2, h->buf.nu2, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(dnu, h->buf.nu2, 2 * sizeof(double), cudaMemcpyDefault, st);
         }
         if (e == cudaSuccess && dtc)
@@ -1177,8 +1177,8 @@ int mr_plate_nu(mr_handle h, double* nu2, mr_stream stream)
     cudaStream_t st = (cudaStream_t)stream;
     const double zz[2] = {h->zc[0] - h->zf[0], h->zf[h->Nz] - h->zc[h->Nz - 1]};
     cudaError_t e = h->cfg.precision == MR_F64
-                        ? launch_plate_nu<double>(h->g64, (const double*)h->buf.T[h->ic], zz, h->buf.nu2, st)
-                        : launch_plate_nu<float>(h->g32, (const float*)h->buf.T[h->ic], zz, h->buf.nu2, st);
+                        ? launch_plate_nu<double>(h->g64, (const double*)h->buf.T[h->ic], zz, h->buf.nu2, h->buf.nu2, st)
+                        : launch_plate_nu<float>(h->g32, (const float*)h->buf.T[h->ic], zz, h->buf.nu2, h->buf.nu2, st);
     if (e != cudaSuccess) return cuda_check(e, "mr_plate_nu: launch");
     return cuda_check(cudaMemcpyAsync(nu2, h->buf.nu2, 2 * sizeof(double), cudaMemcpyDefault, st), "mr_plate_nu: copy");
 }
@@ -1212,10 +1212,9 @@ static double column_volume(mr_handle h)
     return v * (double)h->Nx * (double)h->Nys;
 }
 
-// Volume moments of a dense field in the handle's precision into the handle's results.
-static cudaError_t launch_field_moments(mr_handle h, const void* T, cudaStream_t st)
+// Volume moments of a dense field in the handle's precision into res[0..2].
+static cudaError_t launch_field_moments(mr_handle h, const void* T, double* res, cudaStream_t st)
 {
-    double* const res = h->buf.mom + 1 + 6 * (size_t)kMomentBlocks;
     return h->cfg.precision == MR_F64
                ? launch_moments<double>(h->g64, (const double*)T, h->g64.dz, column_volume(h), h->buf.mom, res, st)
                : launch_moments<float>(h->g32, (const float*)T, h->g64.dz, column_volume(h), h->buf.mom, res, st);
@@ -1246,10 +1245,10 @@ int mr_scalar_stats(mr_handle h, mr_stats* out, mr_stream stream)
     // on the velocity alone: once per velocity
     const bool div = h->have_velocity && !h->maxdiv_valid;
     int n = 0;
-    cudaError_t e = launch_field_moments(h, T, st);
+    cudaError_t e = launch_field_moments(h, T, h->buf.mom + 1 + 6 * (size_t)kMomentBlocks, st);
     if (e == cudaSuccess)
-        e = h->cfg.precision == MR_F64 ? launch_plate_nu<double>(h->g64, (const double*)T, zz, h->buf.nu2, st)
-                                       : launch_plate_nu<float>(h->g32, (const float*)T, zz, h->buf.nu2, st);
+        e = h->cfg.precision == MR_F64 ? launch_plate_nu<double>(h->g64, (const double*)T, zz, h->buf.nu2, h->buf.nu2, st)
+                                       : launch_plate_nu<float>(h->g32, (const float*)T, zz, h->buf.nu2, h->buf.nu2, st);
     if (e == cudaSuccess && div) e = launch_velocity_max(h, 1, &n, st);
     if (e != cudaSuccess) return cuda_check(e, "mr_scalar_stats: launch");
     double res[8];
@@ -1314,30 +1313,6 @@ namespace {
 
 using namespace mr;
 
-// FP64 volume mean and variance of a dense field in precision P.
-int field_moments(mr_handle h, const void* T, double* mean, double* var, cudaStream_t st)
-{
-    double res[3];
-    cudaError_t e = launch_field_moments(h, T, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(res, h->buf.mom + 1 + 6 * (size_t)kMomentBlocks, sizeof res, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    const double v = column_volume(h);
-    *mean = res[0] / v;
-    *var = res[1] / v;
-    return cuda_check(e, "moments");
-}
-
-int field_nu(mr_handle h, const void* T, double nu[2], cudaStream_t st)
-{
-    const double zz[2] = {h->zc[0] - h->zf[0], h->zf[h->Nz] - h->zc[h->Nz - 1]};
-    cudaError_t e = h->cfg.precision == MR_F64 ? launch_plate_nu<double>(h->g64, (const double*)T, zz, h->buf.nu2, st)
-                                               : launch_plate_nu<float>(h->g32, (const float*)T, zz, h->buf.nu2, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(nu, h->buf.nu2, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return cuda_check(e, "plate Nusselt");
-}
-
 cudaError_t step_buffers(mr_handle h, const void* Tm1, const void* T, void* Tp1, int64_t s, cudaStream_t st)
 {
     const StepCoef c = step_coef(h->cfg, s);
@@ -1400,6 +1375,14 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
         a.cp_pairs = cpairs;
         a.ck = ck;
     }
+    if (a.res_levels < nsteps + 1) {
+        if (a.res) dev_free(a.res);
+        a.res = nullptr;
+        a.res_levels = 0;
+        e = dev_malloc((void**)&a.res, 5 * ((size_t)nsteps + 1) * sizeof(double));
+        if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: loss");
+        a.res_levels = nsteps + 1;
+    }
     a.ready = false;
     a.S = nsteps;
     a.ck = ck;
@@ -1417,23 +1400,33 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
             if (e == cudaSuccess) e = cudaMemcpyAsync(pair + fb, Tc, fb, cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: checkpoint");
         }
+        // the level's share of the loss stays on the device until the run has been launched
+        double* const r = a.res + 5 * s;
+        const double zz[2] = {h->zc[0] - h->zf[0], h->zf[h->Nz] - h->zc[h->Nz - 1]};
+        if (a.wnu[s] != 0.0)
+            e = h->cfg.precision == MR_F64
+                    ? launch_plate_nu<double>(h->g64, (const double*)Tc, zz, h->buf.nu2, r, st)
+                    : launch_plate_nu<float>(h->g32, (const float*)Tc, zz, h->buf.nu2, r, st);
+        if (e == cudaSuccess && a.wvar[s] != 0.0) e = launch_field_moments(h, Tc, r + 2, st);
+        if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: loss");
         int rc;
-        if (a.wnu[s] != 0.0) {
-            double nu[2];
-            if ((rc = field_nu(h, Tc, nu, st))) return rc;
-            L += a.wnu[s] * nu[0];
-        }
-        if (a.wvar[s] != 0.0) {
-            double mean = 0.0, var = 0.0;
-            if ((rc = field_moments(h, Tc, &mean, &var, st))) return rc;
-            a.mean[s] = mean;
-            L += a.wvar[s] * var;
-        }
         if (s < nsteps && (rc = mr_scalar_step(h, 1, stream))) return rc;
+    }
+    std::vector<double> res(5 * ((size_t)nsteps + 1));
+    e = cudaMemcpyAsync(res.data(), a.res, res.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward");
+    const double vol = column_volume(h);
+    for (int64_t s = 0; s <= nsteps; ++s) {
+        if (a.wnu[s] != 0.0) L += a.wnu[s] * res[5 * s];
+        if (a.wvar[s] != 0.0) {
+            a.mean[s] = res[5 * s + 2] / vol;
+            L += a.wvar[s] * (res[5 * s + 3] / vol);
+        }
     }
     *loss = L;
     a.ready = true;
-    return cuda_check(cudaStreamSynchronize(st), "mr_adjoint_forward");
+    return MR_OK;
 }
 
 int mr_adjoint_backward(mr_handle h, double gscale, void* gT0, int32_t gT0_dtype, double* gU, double* gV, double* gW,

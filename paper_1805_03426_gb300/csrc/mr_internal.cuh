@@ -187,6 +187,8 @@ struct mr_handle_s {
         float* face32 = nullptr;               // MR_F32: per-segment FP32 sums, flushed into face
         double* scr = nullptr;                 // work of the refinement's transpose, FP64
         double* out = nullptr;                 // FP64 staging of the outputs (dense T0, coarse U, V, W)
+        double* res = nullptr;                 // per level: plate Nusselt numbers (2), volume moments (3)
+        int64_t res_levels = 0;
     } adj;
 };
 
@@ -248,7 +250,7 @@ cudaError_t launch_profiles(const Grid<P>& g, const P* T, const P* Ws, const flo
 // res[3..4] = nu2, res[5] = maximum of part[0..n), res[6] = *err (then cleared); each may be NULL
 cudaError_t launch_gather(const double* nu2, const double* part, int n, int* err, double* res, cudaStream_t st);
 template <typename P>
-cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* out2,
+cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* work, double* out2,
                             cudaStream_t st);
 template <typename P>
 cudaError_t launch_maxdiv(const Grid<P>& g, const P* Us, const P* Vs, const P* Ws, double* partials,

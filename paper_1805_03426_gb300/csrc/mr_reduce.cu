@@ -214,12 +214,13 @@ __global__ void k_convert(const S* __restrict__ src, D* __restrict__ dst, size_t
 }  // namespace
 
 template <typename P>
-cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* out2, cudaStream_t st)
+cudaError_t launch_plate_nu(const Grid<P>& g, const P* T, const double* zb_zt, double* work, double* out2,
+                            cudaStream_t st)
 {
-    // out2 holds 3 + 2 * kPlateBlocks doubles: the two means, the block count
-    // (zero between launches) and the partials
-    k_plate_nu<P><<<kPlateBlocks, 256, 0, st>>>(g, T, zb_zt[0], zb_zt[1], 1.0 / ((double)g.Nx * g.Ny), out2 + 3,
-                                                reinterpret_cast<unsigned*>(out2 + 2), out2);
+    // work holds 3 + 2 * kPlateBlocks doubles: two for a caller's result, the block
+    // count (zero between launches) and the partials
+    k_plate_nu<P><<<kPlateBlocks, 256, 0, st>>>(g, T, zb_zt[0], zb_zt[1], 1.0 / ((double)g.Nx * g.Ny), work + 3,
+                                                reinterpret_cast<unsigned*>(work + 2), out2);
     return cudaGetLastError();
 }
 
@@ -274,7 +275,8 @@ cudaError_t launch_convert(const void* src, int sd, void* dst, int dd, size_t n,
 }
 
 #define MR_INST(P)                                                                                           \
-    template cudaError_t launch_plate_nu<P>(const Grid<P>&, const P*, const double*, double*, cudaStream_t);    \
+    template cudaError_t launch_plate_nu<P>(const Grid<P>&, const P*, const double*, double*, double*,              \
+                                             cudaStream_t);                                                  \
     template cudaError_t launch_maxdiv<P>(const Grid<P>&, const P*, const P*, const P*, double*, int,          \
                                           cudaStream_t);                                                     \
     template cudaError_t launch_cfl<P>(const Grid<P>&, const P*, const P*, const P*, double*, int, cudaStream_t);    \
