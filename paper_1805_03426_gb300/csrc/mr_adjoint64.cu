@@ -16,7 +16,7 @@
 // the coarse gradients cancel to 1e-4 of themselves, so that a product error
 // relative to the warp's largest M would show there.  That leaves 26 FP64 instructions
 // per cell (23 and 2.6 conversions), which is what bounds it: the FP64 pipes are 80 %
-// busy while it runs.  128 x 128 x 96 cells 92 us per step, 130 us in FP64 arithmetic
+// busy while it runs.  128 x 128 x 96 cells 82 us per step, 130 us in FP64 arithmetic
 // throughout.  Rows x blocks per SM on the 40-step gradient: 2 x 4 8.6 ms, 3 x 3 8.6,
 // 2 x 3 8.9, 1 x 6 9.6, 2 x 5 (spills) 9.6, before the layers' gradient factors moved
 // to shared memory and comparisons to integers (2 x 4: 7.3).
@@ -104,11 +104,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_adj_fix(const Args A)
     }
     __syncthreads();
 
-    const int nxt = (g.Nx + kCols - 1) / kCols;
-    const int wid = blockIdx.x * kWarps + (threadIdx.x >> 5);
-    const int j0 = (wid / nxt) * R, i = (wid % nxt) * kCols - 1 + lane;
-    if (j0 >= g.Ny) return;                               // whole warps; no barrier below
-    const bool mine = lane >= 1 && lane <= kCols && i < g.Nx;
+    // the warp's part of the line of all bands of R rows (band_span)
+    const int wid = blockIdx.x * kWarps + (threadIdx.x >> 5), span = band_span(g.Nx), bands = (g.Ny + R - 1) / R;
+    if (wid * kCols >= (bands - 1) * span + g.Nx) return;          // whole warps; no barrier below
+    const int at0 = wid * kCols + lane, band = min(at0 / span, bands - 1), i = at0 - band * span - 1, j0 = band * R;
+    const bool mine = lane >= 1 && lane <= kCols && i >= 0 && i < g.Nx;
     const int ic = WALLS ? min(max(i, 0), g.Nx - 1) : (i + g.Nx) % g.Nx;
     // byte offsets in a plane: rows j0-1 .. j0+R; U rows; V faces j0 .. j0+R
     unsigned ro[R + 2], uo[R], vo[R + 1];
@@ -346,7 +346,8 @@ cudaError_t launch_adj_fix(const Grid<double>& g, const double* Us, const double
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(k), smem, &done[2 * (g.walls != 0) + euler]);
     if (e != cudaSuccess) return e;
     // the chunks of layers that give the shortest run (as in the forward step)
-    const long long nxt = (g.Nx + kCols - 1) / kCols, nyt = (g.Ny + R - 1) / R, blocks = (nxt * nyt + kWarps - 1) / kWarps;
+    const long long line = (long long)((g.Ny + R - 1) / R - 1) * band_span(g.Nx) + g.Nx;
+    const long long blocks = (line + kCols * kWarps - 1) / (kCols * kWarps);
     const long long slots = 152LL * kBlocks;
     double best = 1e300;
     for (int n = (g.Nz + kMaxChunk - 1) / kMaxChunk; n <= g.Nz; ++n) {

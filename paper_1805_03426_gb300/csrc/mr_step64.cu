@@ -4,7 +4,9 @@
 //
 // A warp marches a column of 30 x 3 cells through a chunk of layers.  Its 32
 // lanes hold the 30 columns and one neighbour on each side, so that x
-// neighbours and the fluxes of shared x faces are shuffles; the rows of T^s and
+// neighbours and the fluxes of shared x faces are shuffles; the bands of three
+// rows lie end to end, so that a warp may hold the end of one and the start of
+// the next (band_span); the rows of T^s and
 // T^{s-1} on the current plane, the plane below of T^{s-1} and the flux through
 // the bottom faces stay in registers from layer to layer.  What a layer reads
 // is copied into shared memory one layer ahead (cp.async, 8 bytes a lane: any
@@ -138,11 +140,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
     }
     __syncthreads();
 
-    const int nxt = (g.Nx + kCols - 1) / kCols;
-    const int wid = blockIdx.x * kWarps + (threadIdx.x >> 5);
-    const int j0 = (wid / nxt) * R, i = (wid % nxt) * kCols - 1 + lane;
-    if (j0 >= g.Ny) return;                               // whole warps; no barrier below
-    const bool mine = lane >= 1 && lane <= kCols && i < g.Nx;
+    // the warp's part of the line of all bands of R rows (band_span)
+    const int wid = blockIdx.x * kWarps + (threadIdx.x >> 5), span = band_span(g.Nx), bands = (g.Ny + R - 1) / R;
+    if (wid * kCols >= (bands - 1) * span + g.Nx) return;          // whole warps; no barrier below
+    const int at0 = wid * kCols + lane, band = min(at0 / span, bands - 1), i = at0 - band * span - 1, j0 = band * R;
+    const bool mine = lane >= 1 && lane <= kCols && i >= 0 && i < g.Nx;
     const int ic = WALLS ? min(max(i, 0), g.Nx - 1) : (i + g.Nx) % g.Nx;
     const bool xin = !WALLS || (i > 0 && i < g.Nx);       // the face west of column i carries a flux
     // byte offsets in a plane (below 2^32: step_fix_fits): rows j0-1 .. j0+R; U rows; V faces j0 .. j0+R
@@ -369,7 +371,8 @@ cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
     // The chunks of layers: as many as give the shortest run, the rounds of
     // resident blocks times the layers of a chunk, each chunk's start counted as
     // kStart layers.
-    const long long nxt = (g.Nx + kCols - 1) / kCols, nyt = (g.Ny + R - 1) / R, blocks = (nxt * nyt + kWarps - 1) / kWarps;
+    const long long line = (long long)((g.Ny + R - 1) / R - 1) * band_span(g.Nx) + g.Nx;
+    const long long blocks = (line + kCols * kWarps - 1) / (kCols * kWarps);
     const long long slots = 152LL * kBlocks;
     double best = 1e300;
     for (int n = (g.Nz + kMaxChunk - 1) / kMaxChunk; n <= g.Nz; ++n) {
