@@ -70,9 +70,10 @@ typedef struct {
                                  dense z faces, z_k = (1 + tanh(g(2k/Nz-1))/tanh g)/2 */
     double ra, pr_or_sc;      /* kappa = (ra * pr_or_sc)^-1/2                  */
     double dt;                /* time step (see mr_cfl_dt / mr_set_dt)        */
-    int32_t precision;        /* MR_F64: FP64 storage and flux arithmetic;
+    int32_t precision;        /* MR_F64: FP64 storage, flux arithmetic in FP64
+                                 or 64-bit fixed point of the same accuracy;
                                  MR_F32: FP32 storage and flux arithmetic.
-                                 Reductions are FP64 in both.                 */
+                                 Reductions are of FP64 accuracy in both.     */
     int32_t velocity_mode;    /* MR_VEL_STORED: dense faces kept in HBM;
                                  MR_VEL_FUSED: every stage of the refinement
                                  inside the step kernel, from the coarse faces;
@@ -240,7 +241,7 @@ int mr_upscale_scalar(mr_handle h, double* Tc, mr_stream stream);
  * plates the conductive flux alone).  nu_T (host, may be NULL): Nu_T =
  * eps_T (Ra Pr)^1/2 = <|grad T|^2>, the volume average of the squared face
  * gradients weighted by each face's dual volume, plates at their Dirichlet
- * values.  FP64; synchronises.  Fused modes refine into temporary dense faces. */
+ * values.  Of FP64 accuracy; synchronises. */
 int mr_scalar_profiles(mr_handle h, double* nu_z, double* nu_T, mr_stream stream);
 
 /* Gradients (hand-written discrete adjoint of the scheme above).
@@ -302,8 +303,8 @@ int mr_set_halo_rows(mr_handle h, const void* below, const void* above, mr_strea
 /* Measurement aid (no counterpart in the paper): the FP64 arithmetic rate of
  * the current device in TFLOP/s (an FMA counts two), from a kernel of
  * independent FMA chains in registers timed with CUDA events on stream (best
- * of three launches after one untimed).  The FP64 stored-velocity step is
- * bound by this rate rather than by HBM.  Synchronises.  Errors: MR_ERR_ARG
+ * of three launches after one untimed).  What is left in FP64 arithmetic (the
+ * adjoint's face gradients, the refinement) is bound by it.  Synchronises.  Errors: MR_ERR_ARG
  * (NULL), MR_ERR_CUDA. */
 int mr_fp64_fma_rate(double* tflops, mr_stream stream);
 
