@@ -319,7 +319,15 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_adj_fix(const Args A)
 
 }  // namespace
 
-bool adj_fix_fits(const Grid<double>& g) { return step_fix_fits(g); }
+// Plane offsets below 2^32 bytes, and enough cells to fill the chip: gradients of 40
+// steps, this kernel against k_adj_step_periodic: 32,768 cells 1.31 and 1.17 ms,
+// 110,592 2.10 and 2.43, 196,608 2.54 and 2.60, 262,144 2.62 and 2.81, 512,000 3.49
+// and 4.37.
+bool adj_fix_fits(const Grid<double>& g)
+{
+    const size_t row = (size_t)(g.ufx > g.Nx ? g.ufx : g.Nx), rows = (size_t)(g.vfy > g.Ny ? g.vfy : g.Ny);
+    return row * rows < (1ull << 29) && !g.order4 && (size_t)g.Nx * g.Ny * g.Nz >= 98304;
+}
 
 cudaError_t launch_adj_fix(const Grid<double>& g, const double* Us, const double* Vs, const double* Ws, const double* T,
                            const double* Tprev, const double* Mn, double* Mc, double* Mp, double s_nu, double s_var,

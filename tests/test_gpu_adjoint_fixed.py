@@ -1,4 +1,4 @@
-"""The FP64 backward step in 64-bit fixed point (grids of 196,608 cells and more)
+"""The FP64 backward step in 64-bit fixed point (grids of 98,304 cells and more)
 against the oracle's discrete adjoint: sizes at the edges of its tiles (30 columns
 x 2 rows, chunks of layers), side walls, zero-flux plates, averaging steps, and
 adjoint fields that fall off by many decades within a tile."""
@@ -60,3 +60,11 @@ def test_adjoint_of_the_last_heat_flux_alone(mr, name):  # noqa: F811
     wnu, wvar = np.zeros(6), np.zeros(6)
     wnu[-1] = 1.0
     _compare(mr, p, 5, 5, wnu, wvar)
+
+
+@pytest.mark.parametrize("walls", [0, 1])
+@pytest.mark.parametrize("ny", [23, 24])
+def test_grids_on_both_sides_of_the_smallest_one(mr, ny, walls):  # noqa: F811
+    # 94,208 cells (FP64 arithmetic) and 98,304
+    p = Problem(32, ny, 16, 2, 2, 2, gamma=1.2, walls=walls, np_average=4, dt=2e-4, ra=1e7)
+    _compare(mr, p, 7, 3, *_weights(7))
