@@ -139,10 +139,8 @@ __global__ void __launch_bounds__(256) k_adj_step(Grid<P> g, const P* __restrict
 // the z weights times 1/dz come from g.lz, and the face-gradient factors
 // gdt A_f / 2 (x, y) and gdt A_z arrive as cx, cy, cz per unit dz.
 template <typename P, bool EULER>
-__global__ void __launch_bounds__(256) k_adj_step_periodic(Grid<P> g, const P* __restrict__ Us,
-                                                           const P* __restrict__ Vs, const P* __restrict__ Ws,
-                                                           const P* __restrict__ T, const P* __restrict__ Tprev,
-                                                           const P* __restrict__ Mn, P* __restrict__ Mc,
+__global__ void __launch_bounds__(256) k_adj_step_periodic(Grid<P> g, const P* Us, const P* Vs, const P* Ws,
+                                                           const P* T, const P* Tprev, const P* Mn, P* __restrict__ Mc,
                                                            P* __restrict__ Mp, double s_nu, double s_var,
                                                            double mean_prev, P* __restrict__ gU, P* __restrict__ gV,
                                                            P* __restrict__ gW, P a, P b, P gdt, P cx, P cy, P cz)
@@ -194,10 +192,9 @@ __global__ void __launch_bounds__(256) k_adj_step_periodic(Grid<P> g, const P* _
 __device__ __forceinline__ float get(const float4& v, int q) { return q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w)); }
 __device__ __forceinline__ void put(float4& v, int q, float x) { (q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w))) = x; }
 template <bool EULER>
-__global__ void __launch_bounds__(128) k_adj_step_periodic4(Grid<float> g, const float* __restrict__ Us,
-                                                            const float* __restrict__ Vs, const float* __restrict__ Ws,
-                                                            const float* __restrict__ T, const float* __restrict__ Tprev,
-                                                            const float* __restrict__ Mn, float* __restrict__ Mc,
+__global__ void __launch_bounds__(128) k_adj_step_periodic4(Grid<float> g, const float* Us, const float* Vs,
+                                                            const float* Ws, const float* T, const float* Tprev,
+                                                            const float* Mn, float* __restrict__ Mc,
                                                             float* __restrict__ Mp, double s_nu, double s_var,
                                                             double mean_prev, float* __restrict__ gU, float* __restrict__ gV,
                                                             float* __restrict__ gW, float a, float b, float gdt, float cx,

@@ -1231,8 +1231,8 @@ cudaError_t launch_fl_any(const Grid<float>& g, const FusedInputs& in, const flo
 // conversion and a padding).
 // A thread takes a padded row (component, layer, row) along x: one division per
 // row, coalesced columns.
-__global__ void __launch_bounds__(256) k_pad_coarse64(const double* __restrict__ U, const double* __restrict__ V,
-                                                      const double* __restrict__ W, float* __restrict__ out,
+__global__ void __launch_bounds__(256) k_pad_coarse64(const double* U, const double* V, const double* W,
+                                                      float* __restrict__ out,
                                                       float* __restrict__ U32, float* __restrict__ V32,
                                                       float* __restrict__ W32, int nx, int nyg, int nz, int j0, int ny)
 {
@@ -1287,7 +1287,7 @@ __device__ __forceinline__ double cr_block_sum(double v, double* s)
     return v;
 }
 __global__ void __launch_bounds__(kCRThreads)
-k_coupled_nu(const float* __restrict__ T, size_t plane, size_t top, double izb, double izt, double inv_plane,
+k_coupled_nu(const float* T, size_t plane, size_t top, double izb, double izt, double inv_plane,
              double* __restrict__ work, double* __restrict__ nu2)
 {
     after_previous();

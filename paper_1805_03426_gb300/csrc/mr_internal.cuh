@@ -17,8 +17,11 @@ namespace mr {
 // after_previous() until everything before it has finished and is visible.  Nothing
 // the stream's earlier kernels write is touched before that call, nothing they read
 // is written, and let_next() comes after it, so that a kernel never runs beside one
-// more than one launch ahead.  What this hides is the launch latency and the blocks'
-// start, about 2 us per launch back to back.
+// more than one launch ahead.  Data that the kernel before may write is not read-only
+// for the whole life of such a kernel, so its inputs are not `const __restrict__`,
+// which would let the compiler use the non-coherent loads that require this.  What the
+// early start hides is the launch latency and the blocks' start, about 2 us per launch
+// back to back.
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... K, typename... A>

@@ -18,8 +18,8 @@ constexpr double kTTop = -0.5;
 // levels (temporal refinement, Section 3.4).
 template <typename P, bool LERP>
 struct FaceVel {
-    const P* __restrict__ A;
-    const P* __restrict__ B;
+    const P* A;
+    const P* B;
     P alpha;
     __device__ __forceinline__ P operator[](size_t f) const
     {
@@ -33,7 +33,7 @@ struct FaceVel {
 // f-2 .. f+1 at T[base + c * stride] with the grid's weights; periodic cells
 // wrap, cells beyond a wall carry zero weight and are not read.
 template <typename P>
-__device__ __forceinline__ P face4(const P* __restrict__ w, int f, int N, bool periodic, const P* __restrict__ T,
+__device__ __forceinline__ P face4(const P* w, int f, int N, bool periodic, const P* T,
                                    size_t base, size_t stride)
 {
     P s = 0;
@@ -53,8 +53,7 @@ __device__ __forceinline__ P face4(const P* __restrict__ w, int f, int N, bool p
 template <typename P, bool IMPLZ, bool LERP, bool O4>
 __global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P, LERP> Us,
                                                      const FaceVel<P, LERP> Vs, const FaceVel<P, LERP> Ws,
-                                                     const P* __restrict__ Tm1, const P* __restrict__ T,
-                                                     P* __restrict__ Tp1, P a, P b, P gdt)
+                                                     const P* Tm1, const P* T, P* __restrict__ Tp1, P a, P b, P gdt)
 {
     after_previous();
     let_next();
@@ -135,10 +134,8 @@ __global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P,
 // neighbours are summed before kx2, ky2, and the diagonal and the plate
 // terms come from the per-layer table g.lz.  LF: a plain leapfrog step.
 template <typename P, bool LF>
-__global__ void __launch_bounds__(256) k_step_periodic(Grid<P> g, const P* __restrict__ Us,
-                                                       const P* __restrict__ Vs, const P* __restrict__ Ws,
-                                                       const P* __restrict__ Tm1, const P* __restrict__ T,
-                                                       P* __restrict__ Tp1, P a, P b, P gdt)
+__global__ void __launch_bounds__(256) k_step_periodic(Grid<P> g, const P* Us, const P* Vs, const P* Ws,
+                                                       const P* Tm1, const P* T, P* __restrict__ Tp1, P a, P b, P gdt)
 {
     after_previous();
     let_next();
@@ -180,9 +177,8 @@ constexpr int kMarch = 4;
 __device__ __forceinline__ float get(const float4& v, int q) { return q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w)); }
 __device__ __forceinline__ void put(float4& v, int q, float x) { (q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w))) = x; }
 template <bool LF>
-__global__ void __launch_bounds__(128) k_step_periodic4(Grid<float> g, const float* __restrict__ Us,
-                                                        const float* __restrict__ Vs, const float* __restrict__ Ws,
-                                                        const float* __restrict__ Tm1, const float* __restrict__ T,
+__global__ void __launch_bounds__(128) k_step_periodic4(Grid<float> g, const float* Us, const float* Vs,
+                                                        const float* Ws, const float* Tm1, const float* T,
                                                         float* __restrict__ Tp1, float a, float b, float gdt, int march)
 {
     after_previous();
@@ -417,7 +413,7 @@ cudaError_t step_stored(const Grid<P>& g, const FaceVel<P, LERP>& u, const FaceV
                         grd, blk, 0, st, g, u, v, w, Tm1, T, Tp1, a, b, gdt);
 }
 
-__global__ void k_lerp(const float* __restrict__ A, const float* __restrict__ B, float alpha, float* __restrict__ out,
+__global__ void k_lerp(const float* A, const float* B, float alpha, float* __restrict__ out,
                        size_t n)
 {
     after_previous();
