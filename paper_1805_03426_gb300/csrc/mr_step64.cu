@@ -65,7 +65,7 @@ constexpr int kFieldLo = 1023 - 300, kFieldHi = 1023 + 300;
 
 // The constants of the layers of a block's chunk, scaled by 2^(62 - eR).
 struct LayerK {
-    Bal hz, cdn, cup, ndiag;         // 2 S_W / dz_k, cdn, cup, -(2 kx2 + 2 ky2 + cdn + cup)
+    Bal hz, cdn, cup, ndiag;         // 2 S_W / dz_k, cdn, cup, minus the sum of all neighbours' rates
     Bal wlo, whi;                    // weights of the layer's top face, times 2^62
 };
 
@@ -121,12 +121,16 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
     if (usable) {
         for (int q = threadIdx.x; q < k1 - k0; q += blockDim.x) {
             const int k = k0 + q;
-            const double p = pow2(62 - eR), cdn = A.zs * g.cdn[k], cup = A.zs * g.cup[k];
+            const double p = pow2(62 - eR);
+            // the diagonal is minus the sum of the neighbours' integers, so that the
+            // diffusion of a constant is zero exactly
+            const long long kx = __double2ll_rn(g.kx2 * p), ky = __double2ll_rn(g.ky2 * p);
+            const long long dn = __double2ll_rn(A.zs * g.cdn[k] * p), up = __double2ll_rn(A.zs * g.cup[k] * p);
             LayerK L;
             L.hz = fixed(2.0 * g.inv_dz[k] * pow2(EW - 1022 + 62 - eR));
-            L.cdn = fixed(cdn * p);
-            L.cup = fixed(cup * p);
-            L.ndiag = fixed(-((2.0 * g.kx2 + 2.0 * g.ky2 + cdn + cup) * p));
+            L.cdn = bal(dn);
+            L.cup = bal(up);
+            L.ndiag = bal(-(2 * (kx + ky) + dn + up));
             L.wlo = fixed(g.wlo[k + 1] * 0x1p62);
             L.whi = fixed(g.whi[k + 1] * 0x1p62);
             sk[q] = L;
@@ -265,8 +269,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
         }
         if (plain) {
             // FP64 arithmetic with the same shared fluxes; the bottom faces' are
-            // carried from a layer below that was stepped in the same way
+            // carried from a layer below that was stepped in the same way.  Diffusion
+            // by differences, as k_step_stored has it, but for the periodic explicit
+            // form, which is k_step_periodic's
             const double cdn = A.zs * g.cdn[k], cup = A.zs * g.cup[k];
+            const bool folded = !WALLS && A.zs == 1.0;
             const double ndiag = -2.0 * (g.kx2 + g.ky2) - cdn - cup;
             double xt[R];
 #pragma unroll
@@ -289,13 +296,15 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
                 double fw = s[(kU + r) * 32] * (__shfl_up_sync(0xffffffffu, xt[r], 1) + xt[r]);
                 if (WALLS && !xin) fw = 0.0;
                 const double fe = __shfl_down_sync(0xffffffffu, fw, 1);
-                const double dx = __shfl_up_sync(0xffffffffu, xd[r], 1) + __shfl_down_sync(0xffffffffu, xd[r], 1);
+                const double dw = __shfl_up_sync(0xffffffffu, xd[r], 1), de = __shfl_down_sync(0xffffffffu, xd[r], 1);
                 const double tn = r + 1 < R ? xt[r + 1 < R ? r + 1 : r] : hn, dn = r + 1 < R ? xd[r + 1 < R ? r + 1 : r] : en;
                 double fn = s[(kV + r + 1) * 32] * (xt[r] + tn);
                 if (WALLS && j0 + r + 1 >= g.Ny) fn = 0.0;
                 const double ft = top ? 0.0 : s[(kW + r) * 32] * (g.wlo[k + 1] * xt[r] + g.whi[k + 1] * rt[r]);
                 const double below = k > 0 ? *at(pd - plane, ro[r + 1]) : pl;
-                const double D = g.kx2 * dx + g.ky2 * (ds + dn) + cdn * below + cup * rd[r] + ndiag * xd[r];
+                const double D = folded ? g.kx2 * (dw + de) + g.ky2 * (ds + dn) + cdn * below + cup * rd[r] + ndiag * xd[r]
+                                        : g.kx2 * ((de - xd[r]) - (xd[r] - dw)) + g.ky2 * ((dn - xd[r]) - (xd[r] - ds)) +
+                                              cup * (rd[r] - xd[r]) - cdn * (xd[r] - below);
                 const double sum = g.hx * (fw - fe) + g.hy * (fs - fn) + g.inv_dz[k] * (__longlong_as_double(fb[r]) - ft) + D;
                 if (mine && j0 + r < g.Ny)
                     *const_cast<double*>(at(A.out + (size_t)k * plane, ro[r + 1])) =
