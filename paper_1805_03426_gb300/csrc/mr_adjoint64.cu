@@ -36,6 +36,7 @@ constexpr int kBlocks = 4;           // resident blocks per SM
 constexpr int kStart = 3;            // a chunk's start, in layers
 constexpr int kSpan = 6;             // binades below the warp's largest value that a lane may lie
 constexpr int kMaxChunk = 32;        // layers per chunk
+constexpr int kMaxRate = 7;          // binades that the step's rates gdt 2^eR may reach (mr_step64.cu; a stable step: 2^7)
 constexpr int kFieldLo = 1023 - 300, kFieldHi = 1023 + 300;   // exponent fields of scales
 
 // The constants of the layers of a block's chunk, scaled by 2^(62 - eR), and the
@@ -82,8 +83,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_adj_fix(const Args A)
         m = __reduce_max_sync(0xffffffffu, m);
         const double r = __hiloint2double((int)m + 1, 0) + 4.0 * (g.hx * pow2(EU - 1022) + g.hy * pow2(EV - 1022)) +
                          4.0 * (g.kx2 + g.ky2);
-        eR = ((__double2hiint(r) >> 20) & 0x7ff) - 1022;  // 2^eR > r
-        usable = usable && eR > -400 && eR < 400;
+        eR = exponent(r);                                 // 2^eR > r
+        usable = usable && eR > -400 && eR < 400 && exponent(A.gdt) + eR <= kMaxRate;
     }
     for (int q = threadIdx.x; q < k1 - k0; q += blockDim.x) {
         const int k = k0 + q;

@@ -100,6 +100,9 @@ __device__ __forceinline__ long long dec(double v, int E)
     return fix::dec<BITS>(__double2hiint(v), __double2loint(v), E);
 }
 
+// the least e with v < 2^e, v positive and normal
+__device__ __forceinline__ int exponent(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1022; }
+
 // 2^-900 <= v < 2^900, without an FP64 comparison
 __device__ __forceinline__ bool ordinary(double v)
 {

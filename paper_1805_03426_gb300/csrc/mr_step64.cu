@@ -41,7 +41,12 @@
 // (and not all zero), or which holds an infinity, a NaN or only values near the
 // underflow limit, is stepped in FP64 arithmetic instead (22 operations per cell:
 // a field that falls off by many decades from cell to cell everywhere runs at
-// 0.71 ms, one of zeros and ones at 0.30 ms).
+// 0.71 ms, one of zeros and ones at 0.30 ms).  So is every layer where gdt 2^eR
+// exceeds 2^kMaxRate = 64: a stable explicit step's rates are below 16 (2^eR is up
+// to four times their sum), and beyond the limit the products' error, 2^-58 of
+// them, would pass FP64's rounding -- a single face velocity far above all others
+// with a time step that follows the others, or implicit vertical diffusion over
+// layers much thinner than the time step needs.
 #include <math.h>
 
 #include "mr_fix.cuh"
@@ -59,6 +64,7 @@ constexpr int kBlocks = 4;           // resident blocks per SM
 constexpr int kStart = 3;            // a chunk's start, in layers
 constexpr int kSpan = 6;             // binades below the warp's largest value that a lane may lie
 constexpr int kMaxChunk = 32;        // layers per chunk
+constexpr int kMaxRate = 6;          // binades that the step's rates gdt 2^eR may reach
 // exponent fields of scales: what is smaller or larger (but zero) is left to
 // FP64 arithmetic, so that no power of two below leaves the normal range
 constexpr int kFieldLo = 1023 - 300, kFieldHi = 1023 + 300;
@@ -115,8 +121,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
         m = __reduce_max_sync(0xffffffffu, m);
         const double r = __hiloint2double((int)m + 1, 0) + 4.0 * (g.hx * pow2(EU - 1022) + g.hy * pow2(EV - 1022)) +
                          4.0 * (g.kx2 + g.ky2);
-        eR = ((__double2hiint(r) >> 20) & 0x7ff) - 1022;  // 2^eR > r
-        usable = usable && eR > -400 && eR < 400;
+        eR = exponent(r);                                 // 2^eR > r
+        usable = usable && eR > -400 && eR < 400 && exponent(A.gdt) + eR <= kMaxRate;
     }
     if (usable) {
         for (int q = threadIdx.x; q < k1 - k0; q += blockDim.x) {
