@@ -122,7 +122,7 @@ typedef struct {
     double nu_bot;    /* <(0.5 - T(z_c0)) / z_c0>_xy: bottom-plate Nusselt number  */
     double nu_top;    /* <(T(z_cN-1) + 0.5) / (1 - z_cN-1)>_xy: top-plate Nusselt  */
     double mean;      /* volume-weighted mean of T                                 */
-    double var;       /* volume-weighted variance of T (two-pass)                  */
+    double var;       /* volume-weighted variance of T, about the mean             */
     double integral;  /* sum of T * cell volume                                    */
     double max_div;   /* max over dense cells of |sum of outward face fluxes|/volume
                          of the refined velocity (Section 3.2 divergence check)   */

@@ -164,13 +164,54 @@ __device__ __forceinline__ void moments_unit(const P* __restrict__ r, size_t lo,
     for (; m < hi; m += kThreads) one(r[m]);
 }
 
+// A value near the mean of a unit, in every thread: the mean of kGroup samples per
+// thread spread over it (finite ones; 0 without any).  Whatever the samples miss or
+// hit, the squares about it are at most units / samples (8) times those about the
+// unit's mean, so that at most three bits of them cancel; about one cell's value an
+// outlier just there would cost as many bits as the unit has.
+template <typename P>
+__device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_t hi)
+{
+    constexpr int kGroup = 8;
+    __shared__ P sum[kThreads / 32];
+    __shared__ int num[kThreads / 32];
+    const size_t step = (hi - lo) / kGroup;
+    P s = P(0);
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < kGroup; ++q) {
+        const size_t m = lo + q * step + threadIdx.x;
+        const P t = m < hi ? r[m] : P(NAN);
+        if (isfinite(t)) {
+            s += t;
+            ++n;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) {
+        sum[threadIdx.x >> 5] = s;
+        num[threadIdx.x >> 5] = n;
+    }
+    __syncthreads();
+    s = P(0);
+    n = 0;
+    for (int w = 0; w < kThreads / 32; ++w) {
+        s += sum[w];
+        n += num[w];
+    }
+    __syncthreads();                                      // sum, num are reused
+    const P c = s / P(n > 0 ? n : 1);
+    return isfinite(c) ? c : P(0);
+}
+
 // Sum of T vol and of (T - mean)^2 vol (vol = dz_k, in FP64; the host applies dx dy), the
-// count of non-finite values and their sum of squares into out[0..3].  Every
-// block takes T relative to a value c of its own, so that its squares do not
-// cancel where the scalar varies little about its mean; the block that finishes
-// last (an atomic count, nothing waits) combines the blocks' (sum, squares,
-// weight) about the common mean, in a fixed order.
-// 256 x 256 x 192 FP32 cells: 32 us (40 instructions per cell, and the last block's
+// count of non-finite values and their sum of squares into out[0..3].  A unit takes
+// T relative to a value c near its own mean, so that its squares do not cancel;
+// thread 0 refers the units' sums to the c of the block's first one, and the block
+// that finishes last (an atomic count, nothing waits) combines the blocks' (sum,
+// squares, weight) about the common mean, in a fixed order.
+// 256 x 256 x 192 FP32 cells: 34 us (32 about one cell; 40 instructions per cell, and the last block's
 // FP64 combination at the end); a pass for the mean and one for the squares took
 // 2 x 20 us, each with a copy of the partials to the host and a synchronisation.
 template <typename P>
@@ -181,18 +222,16 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
     const size_t plane = (size_t)g.Nx * g.Ny, per = (plane + per_plane - 1) / per_plane;
     const int units = g.Nz * per_plane;
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};              // thread 0: S1, S2, weight, bad, poison
-    P c = P(0);
-    {
-        const int k = blockIdx.x / per_plane;
-        const size_t lo = (size_t)(blockIdx.x % per_plane) * per;
-        if ((int)blockIdx.x < units && lo < plane) c = T[(size_t)k * plane + lo];
-        if (!isfinite(c)) c = P(0);
-    }
+    P cb = P(0);                                          // c of the block's first unit
+    bool first = true;
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
         const int k = u / per_plane;
         const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
         if (lo >= hi) continue;
         const P* r = T + (size_t)k * plane;
+        const P c = near_mean(r, lo, hi);
+        if (first) cb = c;
+        first = false;
         Sum<P> s[2];
         int bad = 0;
         P poison = P(0), big = fabs(c);
@@ -207,29 +246,27 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
         } else {
             block_sum(s, w);
         }
-        if (threadIdx.x == 0) {
-            v[0] = fma(w[0], dz[k], v[0]);
-            v[1] = fma(w[1], dz[k], v[1]);
-            v[2] = fma((double)(hi - lo), dz[k], v[2]);
-        }
-        if (__syncthreads_or(bad)) {                       // the weight less the bad values'
+        double n[2] = {0.0, 0.0};
+        if (__syncthreads_or(bad)) {
             Sum<double> d[2];
-            double n[2];
             d[0].s = (double)bad;
             d[1].s = (double)poison;
             block_sum(d, n);
-            if (threadIdx.x == 0) {
-                v[2] -= n[0] * dz[k];
-                v[3] += n[0];
-                v[4] += n[1];
-            }
+        }
+        if (threadIdx.x == 0) {
+            const double good = (double)(hi - lo) - n[0], d = (double)c - (double)cb;
+            v[0] = fma(fma(d, good, w[0]), dz[k], v[0]);
+            v[1] = fma(fma(d, fma(d, good, 2.0 * w[0]), w[1]), dz[k], v[1]);
+            v[2] = fma(good, dz[k], v[2]);
+            v[3] += n[0];
+            v[4] += n[1];
         }
     }
     __shared__ bool last;
     if (threadIdx.x == 0) {
         double* p = partials + 6 * (size_t)blockIdx.x;
         for (int q = 0; q < 5; ++q) p[q] = v[q];
-        p[5] = (double)c;
+        p[5] = (double)cb;
         __threadfence();                                  // this block's partials before its count
         last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
