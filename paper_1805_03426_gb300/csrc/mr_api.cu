@@ -57,6 +57,20 @@ bool is_device_pointer(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether the handle's kernels may use all three arrays where they lie.
+static bool in_place(mr_handle h, const void* x, const void* y, const void* z)
+{
+    for (const void* p : {x, y, z}) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (!usable_in_place(a, h->device, p)) return false;
+    }
+    return true;
+}
+
 StepCoef step_coef(const mr_config& cfg, int64_t s)
 {
     // Section 2.2: leapfrog, averaging every N_p steps; s = 0 starts with Euler.
@@ -676,7 +690,7 @@ static int load_velocity(mr_handle h, const double* U, const double* V, const do
     DeviceBuffers& b = h->buf;
     int rc;
     const bool f32 = h->cfg.precision == MR_F32;
-    if (f32 && is_device_pointer(U) && is_device_pointer(V) && is_device_pointer(W)) {
+    if (f32 && in_place(h, U, V, W)) {
         // device faces of an FP32 handle: converted from where they are, no FP64 copy
         const double* const src[3] = {U, V, W};
         return derive_velocity(h, src, st);
@@ -898,7 +912,7 @@ int mr_refine_velocity(mr_handle h, const double* U, const double* V, const doub
     // FP64 dense faces given out in device memory are written with the handle's own
     void* const copy[3] = {Us, Vs, Ws};
     const bool stored = h->cfg.velocity_mode == MR_VEL_STORED;
-    const bool direct = Us && stored && h->elt == 8 && is_device_pointer(Us) && is_device_pointer(Vs) && is_device_pointer(Ws);
+    const bool direct = Us && stored && h->elt == 8 && in_place(h, Us, Vs, Ws);
     int rc = load_velocity(h, U, V, W, st, direct ? copy : nullptr);
     if (rc) return rc;
     h->have_velocity = true;

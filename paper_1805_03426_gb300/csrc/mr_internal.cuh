@@ -200,6 +200,14 @@ namespace mr {
 int set_error(int code, const std::string& msg);
 int cuda_check(cudaError_t e, const char* what);
 bool is_device_pointer(const void* p);
+// Whether the kernels of a handle on `device` may read or write FP64 values at p where
+// they lie: device memory of that device (another one's may not be mapped on it) or
+// managed memory, on an 8-byte boundary.  What may not goes through a copy.
+inline bool usable_in_place(const cudaPointerAttributes& a, int device, const void* p)
+{
+    return (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device)) &&
+           reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+}
 StepCoef step_coef(const mr_config& cfg, int64_t s);
 
 // launchers (return cudaError_t of the launch)
