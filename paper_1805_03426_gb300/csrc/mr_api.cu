@@ -510,7 +510,12 @@ int mr_create(const mr_config* cfg, mr_handle* out)
         alloc(&b.Us, h->nU * h->elt);
         alloc(&b.Vs, h->nV * h->elt);
         alloc(&b.Ws, h->nW * h->elt);
-        if (h->elt == 8) alloc((void**)&b.vmax, 4 * sizeof(unsigned));
+        if (h->elt == 8) {
+            alloc((void**)&b.vmax, 4 * sizeof(unsigned));
+        } else {
+            alloc(&b.scrW, (size_t)(h->Nz + 1) * c.ny * c.nx * h->elt);
+            alloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * c.nx * h->elt);
+        }
     }
     const size_t mb64 = metric_bytes<double>(h), mb32 = metric_bytes<float>(h);
     const size_t nwin = 3 * ((size_t)c.nx + c.ny + c.nz);
@@ -582,6 +587,15 @@ int mr_create(const mr_config* cfg, mr_handle* out)
     if (!rc && b.fsc) {
         const std::vector<float> sc = fused_slab_constants(c.nz, c.mz, h->Rz.data(), h->dz.data());
         rc = cuda_check(cudaMemcpy(b.fsc, sc.data(), sc.size() * 4, cudaMemcpyHostToDevice), "mr_create: slab constants");
+    }
+    if (!rc && c.velocity_mode == MR_VEL_STORED && h->elt == 8) {
+        // the refinement's work, in smaller groups of slabs (more launches) where memory is short
+        b.rslabs = refine_slabs(h->g64);
+        while ((e = dev_malloc(&b.rwork, refine_work(h->g64, b.rslabs))) == cudaErrorMemoryAllocation && b.rslabs > 1) {
+            cudaGetLastError();
+            b.rslabs = (b.rslabs + 1) / 2;
+        }
+        rc = cuda_check(e, "mr_create: refinement work");
     }
     if (rc) {
         mr_destroy(h);
@@ -660,12 +674,10 @@ static int refine_into(mr_handle h, void* const dense[3], void* const copy[3], u
     DeviceBuffers& b = h->buf;
     cudaError_t e = cudaSuccess;
     if (h->cfg.precision == MR_F64) {
-        if (!b.rwork) e = dev_malloc(&b.rwork, refine_work(h->g64));
-        if (e != cudaSuccess) return cuda_check(e, "refinement work");
         double* const d[3] = {(double*)dense[0], (double*)dense[1], (double*)dense[2]};
         double* const c[3] = {copy ? (double*)copy[0] : nullptr, copy ? (double*)copy[1] : nullptr,
                               copy ? (double*)copy[2] : nullptr};
-        e = launch_refine<double>(h->g64, b.U64, b.V64, b.W64, d, c, vmax, (double*)b.rwork, st);
+        e = launch_refine<double>(h->g64, b.U64, b.V64, b.W64, d, c, vmax, (double*)b.rwork, b.rslabs, st);
     } else {
         if (!b.scrW) e = dev_malloc(&b.scrW, (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx * h->elt);
         if (e == cudaSuccess && !b.scrV) e = dev_malloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * h->cfg.nx * h->elt);

@@ -98,9 +98,10 @@ struct DeviceBuffers {
     void* Vs = nullptr;
     void* Ws = nullptr;
     unsigned* vmax = nullptr;                  // MR_VEL_STORED, FP64: largest |U|, |V|, |W| (high words)
-    void* rwork = nullptr;                     // FP64: work of the dense refinement (refine_work)
-    void* scrW = nullptr;                      // FP32: full-coarse-area W per dense plane
-    void* scrV = nullptr;                      // FP32: full-coarse-width V per dense row
+    void* rwork = nullptr;                     // MR_VEL_STORED, FP64: work of the refinement (refine_work)
+    int rslabs = 0;                            // coarse slabs that it holds
+    void* scrW = nullptr;                      // FP32: full-coarse-area W per dense plane (lazy in the fused modes)
+    void* scrV = nullptr;                      // FP32: full-coarse-width V per dense row (lazy in the fused modes)
     void* metric = nullptr;                    // one block holding every Grid array
     double* red = nullptr;                     // reduction partials
     double* mom = nullptr;                     // work of the volume moments, then 8 results (launch_gather)
@@ -212,12 +213,15 @@ StepCoef step_coef(const mr_config& cfg, int64_t s);
 
 // launchers (return cudaError_t of the launch)
 // FP64: the dense faces out[3] (and, unless NULL, a second copy of them in copy[3]);
-// vmax (may be NULL): the largest magnitudes of the components; work: refine_work bytes.
+// vmax (may be NULL): the largest magnitudes of the components; work: refine_work bytes
+// for groups of that many coarse slabs (refine_slabs where memory allows, any less do).
 template <typename P>
-size_t refine_work(const Grid<P>& g);
+int refine_slabs(const Grid<P>& g);
+template <typename P>
+size_t refine_work(const Grid<P>& g, int slabs);
 template <typename P>
 cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* const out[3], P* const copy[3],
-                          unsigned* vmax, P* work, cudaStream_t st);
+                          unsigned* vmax, P* work, int slabs, cudaStream_t st);
 // The same with little more memory than the outputs (slower): scrW (Nz + 1) ny nx,
 // scrV Nz (Ny + w) nx values.
 template <typename P>

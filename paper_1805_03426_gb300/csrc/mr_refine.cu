@@ -517,8 +517,11 @@ void launch_coarse(const Refine<P>& A, size_t S, size_t L, cudaStream_t st)
     else k_y_split<P, N, false><<<gy, kThreads, 0, st>>>(A);
     k_row_v<P, N><<<grid(L * g.cvy * g.nx), kThreads, 0, st>>>(A);
 }
+
+}  // namespace
+
 template <typename P>
-int slabs_together(const Grid<P>& g)
+int refine_slabs(const Grid<P>& g)
 {
     size_t n[6];
     int s = g.nz;
@@ -526,19 +529,18 @@ int slabs_together(const Grid<P>& g)
     while (s > 1 && (slab_values(g, n, s) * sizeof(P) > kRefineWork || (size_t)s * g.mz > 65535u * kDenseLayers)) s = (s + 1) / 2;
     return s;
 }
-
-}  // namespace
+template int refine_slabs<double>(const Grid<double>&);
 
 template <typename P>
-size_t refine_work(const Grid<P>& g)
+size_t refine_work(const Grid<P>& g, int slabs)
 {
     size_t n[6];
-    return slab_values(g, n, slabs_together(g)) * sizeof(P);
+    return slab_values(g, n, slabs) * sizeof(P);
 }
 
 template <typename P>
 cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* const out[3], P* const copy[3],
-                          unsigned* vmax, P* work, cudaStream_t st)
+                          unsigned* vmax, P* work, int slabs, cudaStream_t st)
 {
     Refine<P> A;
     A.g = g;
@@ -564,15 +566,14 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
                        &done[form]);
     if (e != cudaSuccess) return e;
     size_t n[6];
-    const int together = slabs_together(g);
-    slab_values(g, n, together);
+    slab_values(g, n, slabs);
     P** const part[6] = {&A.UZ, &A.VZ, &A.WC, &A.UO, &A.WY, &A.VR};
     for (int q = 0; q < 6; ++q) {
         *part[q] = work;
         work += n[q];
     }
     for (A.K0 = 0; A.K0 < g.nz; A.K0 = A.K1) {
-        A.K1 = std::min(A.K0 + together, g.nz);
+        A.K1 = std::min(A.K0 + slabs, g.nz);
         const size_t S = A.K1 - A.K0, L = S * g.mz;
         // 32-bit indexes unless a slab is enormous
         if (slab_values(g, n, (int)S) < (1ull << 31)) launch_coarse<P, unsigned>(A, S, L, st);
@@ -588,9 +589,9 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
     }
     return e;
 }
-template size_t refine_work<double>(const Grid<double>&);
+template size_t refine_work<double>(const Grid<double>&, int);
 template cudaError_t launch_refine<double>(const Grid<double>&, const double*, const double*, const double*,
-                                           double* const[3], double* const[3], unsigned*, double*, cudaStream_t);
+                                           double* const[3], double* const[3], unsigned*, double*, int, cudaStream_t);
 
 template <typename P>
 cudaError_t launch_refine_in_place(const Grid<P>& g, const P* U, const P* V, const P* W, P* Us, P* Vs, P* Ws, P* scrW,
