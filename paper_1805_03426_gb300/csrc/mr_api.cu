@@ -1380,8 +1380,14 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
     auto& a = h->adj;
     const size_t cpairs = (size_t)((nsteps + ck - 1) / ck);
     const size_t fb = h->ncell * h->elt;
-    if (a.cp && (a.cp_pairs < cpairs || a.ck < ck)) adj_free(h);
     cudaError_t e = cudaSuccess;
+    // the levels' results first: refused here, the call has changed nothing
+    double* res_new = nullptr;
+    if (a.res_levels < nsteps + 1) {
+        e = dev_malloc((void**)&res_new, 5 * ((size_t)nsteps + 1) * sizeof(double));
+        if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: loss");
+    }
+    if (a.cp && (a.cp_pairs < cpairs || a.ck < ck)) adj_free(h);
     if (!a.cp) {
         e = dev_malloc(&a.cp, cpairs * 2 * fb);
         if (e == cudaSuccess) e = dev_malloc(&a.seg, ((size_t)ck + 1) * fb);
@@ -1396,17 +1402,15 @@ int mr_adjoint_forward(mr_handle h, int64_t nsteps, int32_t ck, const double* wn
         }
         if (e != cudaSuccess) {
             adj_free(h);
+            dev_free(res_new);
             return cuda_check(e, "mr_adjoint_forward: checkpoint store");
         }
         a.cp_pairs = cpairs;
         a.ck = ck;
     }
-    if (a.res_levels < nsteps + 1) {
-        if (a.res) dev_free(a.res);
-        a.res = nullptr;
-        a.res_levels = 0;
-        e = dev_malloc((void**)&a.res, 5 * ((size_t)nsteps + 1) * sizeof(double));
-        if (e != cudaSuccess) return cuda_check(e, "mr_adjoint_forward: loss");
+    if (res_new) {
+        dev_free(a.res);
+        a.res = res_new;
         a.res_levels = nsteps + 1;
     }
     a.ready = false;
