@@ -239,9 +239,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_adj_fix(const Args A)
             }
         } else {
             const LayerK& L = sk[k - k0];
-            long long ms = dec<59>(hs, E);                // M of the row to the south
             const long long mnh = dec<59>(hn, E);
-            long long ds = m[0] - ms, fs = mul(bal(ds), bal(dec<62>(s[kV * 32], EV)));
+            long long ds = m[0] - dec<59>(hs, E), fs = mul(bal(ds), bal(dec<62>(s[kV * 32], EV)));
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const long long dw = m[r] - __shfl_up_sync(0xffffffffu, m[r], 1);
@@ -273,7 +272,6 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_adj_fix(const Args A)
                 fs = fn;
                 db[r] = d1;
                 qb[r] = qt;
-                ms = m[r];
                 m[r] = mt;
             }
         }

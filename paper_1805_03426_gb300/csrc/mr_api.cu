@@ -521,7 +521,7 @@ int mr_create(const mr_config* cfg, mr_handle* out)
     const size_t nwin = 3 * ((size_t)c.nx + c.ny + c.nz);
     alloc(&b.metric, mb64 + mb32 + (size_t)h->Nz * sizeof(double) + nwin * sizeof(int));
     h->red_blocks = 152 * 8;
-    alloc((void**)&b.red, (size_t)h->red_blocks * 2 * sizeof(double));
+    alloc((void**)&b.red, (size_t)h->red_blocks * sizeof(double));
     alloc((void**)&b.mom, (1 + 6 * (size_t)kMomentBlocks + 8) * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(b.mom, 0, (1 + 6 * (size_t)kMomentBlocks + 8) * sizeof(double));
     alloc((void**)&b.nu2, (3 + 2 * kPlateBlocks) * sizeof(double));
@@ -677,7 +677,7 @@ static int refine_into(mr_handle h, void* const dense[3], void* const copy[3], u
         double* const d[3] = {(double*)dense[0], (double*)dense[1], (double*)dense[2]};
         double* const c[3] = {copy ? (double*)copy[0] : nullptr, copy ? (double*)copy[1] : nullptr,
                               copy ? (double*)copy[2] : nullptr};
-        e = launch_refine<double>(h->g64, b.U64, b.V64, b.W64, d, c, vmax, (double*)b.rwork, b.rslabs, st);
+        e = launch_refine(h->g64, b.U64, b.V64, b.W64, d, c, vmax, (double*)b.rwork, b.rslabs, st);
     } else {
         if (!b.scrW) e = dev_malloc(&b.scrW, (size_t)(h->Nz + 1) * h->cfg.ny * h->cfg.nx * h->elt);
         if (e == cudaSuccess && !b.scrV) e = dev_malloc(&b.scrV, (size_t)h->Nz * (h->Ny + h->w) * h->cfg.nx * h->elt);

@@ -215,13 +215,10 @@ StepCoef step_coef(const mr_config& cfg, int64_t s);
 // FP64: the dense faces out[3] (and, unless NULL, a second copy of them in copy[3]);
 // vmax (may be NULL): the largest magnitudes of the components; work: refine_work bytes
 // for groups of that many coarse slabs (refine_slabs where memory allows, any less do).
-template <typename P>
-int refine_slabs(const Grid<P>& g);
-template <typename P>
-size_t refine_work(const Grid<P>& g, int slabs);
-template <typename P>
-cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* const out[3], P* const copy[3],
-                          unsigned* vmax, P* work, int slabs, cudaStream_t st);
+int refine_slabs(const Grid<double>& g);
+size_t refine_work(const Grid<double>& g, int slabs);
+cudaError_t launch_refine(const Grid<double>& g, const double* U, const double* V, const double* W, double* const out[3],
+                          double* const copy[3], unsigned* vmax, double* work, int slabs, cudaStream_t st);
 // The same with little more memory than the outputs (slower): scrW (Nz + 1) ny nx,
 // scrV Nz (Ny + w) nx values.
 template <typename P>

@@ -249,70 +249,69 @@ constexpr size_t kRefineWork = (size_t)256 << 20;
 // combination of two differences).  SYM: m = 2 on a uniform axis with every window
 // centred on its cell (periodic), whose rows are (1, 8, -1) / 8 and (-1, 8, 1) / 8;
 // known at compile time, or both forms would be computed.
-template <bool SYM, typename P, typename Out>
-__device__ __forceinline__ void split(P c0, P c1, P c2, const P* __restrict__ r, int m, Out out)
+template <bool SYM, typename Out>
+__device__ __forceinline__ void split(double c0, double c1, double c2, const double* __restrict__ r, int m, Out out)
 {
     if constexpr (SYM) {
-        const P d = P(0.125) * (c0 - c2);
+        const double d = 0.125 * (c0 - c2);
         out(0, c1 + d);
         out(1, c1 - d);
         return;
     }
-    const P d0 = c0 - c1, d2 = c2 - c1;
+    const double d0 = c0 - c1, d2 = c2 - c1;
 #pragma unroll
     for (int b = 0; b < m; ++b) out(b, c1 + r[3 * b] * d0 + r[3 * b + 2] * d2);
 }
 
-template <typename P>
 struct Refine {
-    Grid<P> g;
-    const P *U, *V, *W;              // coarse faces
-    P *UZ, *VZ, *WC, *UO, *WY, *VR;  // of the group's slabs K0 .. K1 - 1
-    P *Us, *Vs, *Ws;                 // dense faces
-    P *Ue, *Ve, *We;                 // a second copy of them, or NULL
-    unsigned* vmax;                  // FP64: largest magnitudes of the components, or NULL
+    Grid<double> g;
+    const double *U, *V, *W;         // coarse faces
+    double *UZ, *VZ, *WC, *UO, *WY, *VR;   // of the group's slabs K0 .. K1 - 1
+    double *Us, *Vs, *Ws;            // dense faces
+    double *Ue, *Ve, *We;            // a second copy of them, or NULL
+    unsigned* vmax;                  // largest magnitudes of the components, or NULL
     int K0, K1;
     int layers;                      // of a block of k_dense
-    P iDX, iDY, dydX, dxdy;          // 1 / DX, 1 / DY, dy / DX, dx / dy
+    double iDX, iDY, dydX, dxdy;     // 1 / DX, 1 / DY, dy / DX, dx / dy
 };
 
-template <typename P, typename N>
-__global__ void __launch_bounds__(kThreads) k_z_split(const Refine<P> A)
+template <typename N>
+__global__ void __launch_bounds__(kThreads) k_z_split(const Refine A)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     const N nu = (N)(A.K1 - A.K0) * g.ny * g.cux, nv = (N)(A.K1 - A.K0) * g.cvy * g.nx;
     for (N t = (N)blockIdx.x * blockDim.x + threadIdx.x; t < nu + nv; t += (N)gridDim.x * blockDim.x) {
         const bool u = t < nu;
         const N plane = u ? (N)g.ny * g.cux : (N)g.cvy * g.nx, e = u ? t : t - nu;
         const int q = (int)(e / plane), K = A.K0 + q;
-        const P* src = (u ? A.U : A.V) + e % plane;
-        P* dst = (u ? A.UZ : A.VZ) + (size_t)q * g.mz * plane + e % plane;
+        const double* src = (u ? A.U : A.V) + e % plane;
+        double* dst = (u ? A.UZ : A.VZ) + (size_t)q * g.mz * plane + e % plane;
         if (g.mz == 1) {
             dst[0] = src[(size_t)K * plane];
             continue;
         }
         const int* w = g.wz + 3 * K;
         split<false>(src[(size_t)w[0] * plane], src[(size_t)w[1] * plane], src[(size_t)w[2] * plane],
-                     g.Rz + 3 * (size_t)K * g.mz, g.mz, [&](int b, P v) { dst[(size_t)b * plane] = v; });
+                     g.Rz + 3 * (size_t)K * g.mz, g.mz, [&](int b, double v) { dst[(size_t)b * plane] = v; });
     }
 }
 
-template <typename P, typename N>
-__global__ void __launch_bounds__(kThreads) k_slab_balance(const Refine<P> A)
+template <typename N>
+__global__ void __launch_bounds__(kThreads) k_slab_balance(const Refine A)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     const N plane = (N)g.ny * g.nx, n = (N)(A.K1 - A.K0) * plane;
     for (N t = (N)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (N)gridDim.x * blockDim.x) {
         const int q = (int)(t / plane), K = A.K0 + q;
         const int J = (int)((t % plane) / g.nx), I = (int)(t % g.nx);
         const int Ie = g.walls ? I + 1 : (I + 1 == g.nx ? 0 : I + 1), Jn = g.walls ? J + 1 : (J + 1 == g.ny ? 0 : J + 1);
-        P F = A.W[(size_t)(K + 1) * plane + (t % plane)];
-        P* wc = A.WC + (size_t)q * g.mz * plane + t % plane;
+        double F = A.W[(size_t)(K + 1) * plane + (t % plane)];
+        double* wc = A.WC + (size_t)q * g.mz * plane + t % plane;
         if (K == A.K1 - 1) wc[(size_t)g.mz * plane] = F;
         for (int c = g.mz - 1; c >= 1; --c) {
             const size_t k = (size_t)q * g.mz + c;
-            const P* u = A.UZ + (k * g.ny + J) * g.cux;
-            const P* v = A.VZ + k * g.cvy * g.nx + I;
+            const double* u = A.UZ + (k * g.ny + J) * g.cux;
+            const double* v = A.VZ + k * g.cvy * g.nx + I;
             F += g.dz[K * g.mz + c] * ((u[Ie] - u[I]) * A.iDX + (v[(size_t)Jn * g.nx] - v[(size_t)J * g.nx]) * A.iDY);
             wc[(size_t)c * plane] = F;
         }
@@ -321,10 +320,10 @@ __global__ void __launch_bounds__(kThreads) k_slab_balance(const Refine<P> A)
 }
 
 // R_y of UZ (rows of cux) and WC (rows of nx): thread per (plane, coarse row, column).
-template <typename P, typename N, bool SYM>
-__global__ void __launch_bounds__(kThreads) k_y_split(const Refine<P> A)
+template <typename N, bool SYM>
+__global__ void __launch_bounds__(kThreads) k_y_split(const Refine A)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     const int L = (A.K1 - A.K0) * g.mz;
     const N nu = (N)L * g.ny * g.cux, nw = (N)(L + 1) * g.ny * g.nx;
     for (N t = (N)blockIdx.x * blockDim.x + threadIdx.x; t < nu + nw; t += (N)gridDim.x * blockDim.x) {
@@ -332,37 +331,37 @@ __global__ void __launch_bounds__(kThreads) k_y_split(const Refine<P> A)
         const int row = u ? g.cux : g.nx;
         const N e = u ? t : t - nu, er = e / row;
         const int I = (int)(e - er * row), k = (int)(er / g.ny), J = (int)(er - (N)k * g.ny);
-        const P* src = (u ? A.UZ : A.WC) + (size_t)k * g.ny * row + I;
-        P* dst = (u ? A.UO : A.WY) + ((size_t)k * g.Ny + (size_t)J * g.my) * row + I;
+        const double* src = (u ? A.UZ : A.WC) + (size_t)k * g.ny * row + I;
+        double* dst = (u ? A.UO : A.WY) + ((size_t)k * g.Ny + (size_t)J * g.my) * row + I;
         if (g.my == 1) {
             dst[0] = src[(size_t)J * row];
             continue;
         }
         const int* w = g.wy + 3 * J;
         split<SYM>(src[(size_t)w[0] * row], src[(size_t)w[1] * row], src[(size_t)w[2] * row], g.Ry + 3 * (size_t)J * g.my,
-                   g.my, [&](int b, P v) { dst[(size_t)b * row] = v; });
+                   g.my, [&](int b, double v) { dst[(size_t)b * row] = v; });
     }
 }
 
-template <typename P, typename N>
-__global__ void __launch_bounds__(kThreads) k_row_v(const Refine<P> A)
+template <typename N>
+__global__ void __launch_bounds__(kThreads) k_row_v(const Refine A)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     const int L = (A.K1 - A.K0) * g.mz;
     const N n = (N)L * g.cvy * g.nx;
     for (N t = (N)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (N)gridDim.x * blockDim.x) {
         const N tr = t / g.nx;
         const int I = (int)(t - tr * g.nx), k = (int)(tr / g.cvy), J = (int)(tr - (N)k * g.cvy);
-        P v = A.VZ[t];
-        P* dst = A.VR + ((size_t)k * g.vfy + (size_t)J * g.my) * g.nx + I;
+        double v = A.VZ[t];
+        double* dst = A.VR + ((size_t)k * g.vfy + (size_t)J * g.my) * g.nx + I;
         dst[0] = v;
         if (J == g.ny) continue;                           // the north wall's faces
         const int Ie = g.walls ? I + 1 : (I + 1 == g.nx ? 0 : I + 1);
-        const P dydz = g.dy * g.inv_dz[A.K0 * g.mz + k];
+        const double dydz = g.dy * g.inv_dz[A.K0 * g.mz + k];
         for (int b = 0; b < g.my - 1; ++b) {
             const size_t r = (size_t)k * g.Ny + (size_t)J * g.my + b;
-            const P* u = A.UO + r * g.cux;
-            const P* w = A.WY + r * g.nx + I;
+            const double* u = A.UO + r * g.cux;
+            const double* w = A.WY + r * g.nx + I;
             v = v - (u[Ie] - u[I]) * A.dydX - (w[(size_t)g.Ny * g.nx] - w[0]) * dydz;
             dst[(size_t)(b + 1) * g.nx] = v;
         }
@@ -375,16 +374,16 @@ __global__ void __launch_bounds__(kThreads) k_row_v(const Refine<P> A)
 // memory, where U's cell balance reads them and whole rows are written from.
 constexpr int kDenseRows = 8, kDenseLayers = 8;
 // MX: the refinement in x where known at compile time (2, 4), else 0; SYM: see split.
-template <typename P, int MX, bool SYM>
-__global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P> A)
+template <int MX, bool SYM>
+__global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine A)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     const int mx = MX ? MX : g.mx;
     extern __shared__ __align__(16) unsigned char dsm[];
     const int row = 32 * mx, lane = threadIdx.x & 31, r = threadIdx.x >> 5;
-    P* const wv = reinterpret_cast<P*>(dsm);               // [2][8][row]
-    P* const vv = wv + 2 * kDenseRows * row;               // [2][9][row]
-    P* const uv = vv + 2 * (kDenseRows + 1) * row;         // [8][row]
+    double* const wv = reinterpret_cast<double*>(dsm);     // [2][8][row]
+    double* const vv = wv + 2 * kDenseRows * row;          // [2][9][row]
+    double* const uv = vv + 2 * (kDenseRows + 1) * row;    // [8][row]
     const int ntx = (g.nx + 31) / 32, bx = blockIdx.x % ntx;
     const int I = bx * 32 + lane, j = (blockIdx.x / ntx) * kDenseRows + r;
     const int i0 = bx * row, ni = min(row, g.Nx - i0);
@@ -393,32 +392,29 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
     const bool vrow = col && j <= g.Ny;
     const int jv = (!g.walls && j == g.Ny) ? 0 : j;
     const int w0 = col ? g.wx[3 * I] : 0, w1 = col ? g.wx[3 * I + 1] : 0, w2 = col ? g.wx[3 * I + 2] : 0;
-    const P* const rx = g.Rx + 3 * (size_t)(col ? I : 0) * mx;
+    const double* const rx = g.Rx + 3 * (size_t)(col ? I : 0) * mx;
     unsigned mu = 0, mv = 0, mw = 0;
-    auto mag = [](P v) {
-        if constexpr (sizeof(P) == 8) return (unsigned)__double2hiint(v) & 0x7fffffffu;
-        else return 0u;
-    };
+    auto mag = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
     // the window of this thread's column in a coarse row, and its split along x into a
     // shared row
-    auto window = [&](const P* src, P (&c)[3]) {
+    auto window = [&](const double* src, double (&c)[3]) {
         c[1] = src[mx == 1 ? I : w1];
         if (mx > 1) {
             c[0] = src[w0];
             c[2] = src[w2];
         }
     };
-    auto xsplit = [&](const P (&c)[3], P* dst) {
+    auto xsplit = [&](const double (&c)[3], double* dst) {
         if (mx == 1) dst[lane] = c[1];
-        else split<SYM>(c[0], c[1], c[2], rx, mx, [&](int b, P v) { dst[lane * mx + b] = v; });
+        else split<SYM>(c[0], c[1], c[2], rx, mx, [&](int b, double v) { dst[lane * mx + b] = v; });
     };
     // a shared row to a dense one (and its copy), n values
-    auto put = [&](const P* src, P* a, P* b, size_t at, int n, unsigned& m) {
+    auto put = [&](const double* src, double* a, double* b, size_t at, int n, unsigned& m) {
 #pragma unroll
         for (int q = 0; q < mx; ++q) {
             const int e = lane + 32 * q;
             if (e >= n) break;
-            const P v = src[e];
+            const double v = src[e];
             m = max(m, mag(v));
             a[at + e] = v;
             if (b) b[at + e] = v;
@@ -428,7 +424,7 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
     auto vface = [&](int l, int q) { return vv + ((l & 1) * (kDenseRows + 1) + q) * row; };
     const size_t k00 = (size_t)A.K0 * g.mz;
     // what a layer splits is loaded a layer ahead
-    P cv[3], cw[3], cu = P(0);
+    double cv[3], cw[3], cu = 0.0;
     auto ahead = [&](int l) {
         if (vrow) window(A.VR + ((size_t)l * g.vfy + jv) * g.nx, cv);
         if (own && col) {
@@ -447,7 +443,7 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
     if (l0 < l1) ahead(l0);
     for (int l = l0; l < l1; ++l) {
         const size_t k = k00 + l;
-        P h = cu;
+        double h = cu;
         if (vrow) xsplit(cv, vface(l, r));
         if (own && col) xsplit(cw, wrow(l + 1));
         if (l + 1 < l1) ahead(l + 1);
@@ -457,10 +453,10 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
         if (g.walls && r == kDenseRows && j == g.Ny) put(vface(l, r), A.Vs, A.Ve, (k * g.vfy + j) * g.Nx + i0, ni, mv);
         if (!own) continue;
         put(wrow(l + 1), A.Ws, A.We, ((k + 1) * g.Ny + j) * g.Nx + i0, ni, mw);
-        P* const u = uv + r * row;
+        double* const u = uv + r * row;
         if (col) {
-            const P dxdz = g.dx * g.inv_dz[k];
-            const P *vs = vface(l, r), *vn = vface(l, r + 1), *wb = wrow(l), *wt = wrow(l + 1);
+            const double dxdz = g.dx * g.inv_dz[k];
+            const double *vs = vface(l, r), *vn = vface(l, r + 1), *wb = wrow(l), *wt = wrow(l + 1);
 #pragma unroll
             for (int a = 0; a < mx; ++a) {
                 const int e = lane * mx + a;
@@ -473,7 +469,7 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
         const size_t at = (k * g.Ny + j) * g.ufx + i0;
         put(u, A.Us, A.Ue, at, ni, mu);
         if (g.walls && I == g.nx - 1) {                    // the east wall's face
-            const P v = A.UO[((size_t)l * g.Ny + j) * g.cux + g.nx];
+            const double v = A.UO[((size_t)l * g.Ny + j) * g.cux + g.nx];
             mu = max(mu, mag(v));
             A.Us[at + ni] = v;
             if (A.Ue) A.Ue[at + ni] = v;
@@ -490,8 +486,7 @@ __global__ void __launch_bounds__(32 * (kDenseRows + 1)) k_dense(const Refine<P>
 
 // Values of the intermediates of one coarse slab (refine_work) and how many slabs
 // go together.
-template <typename P>
-size_t slab_values(const Grid<P>& g, size_t (&n)[6], int slabs)
+size_t slab_values(const Grid<double>& g, size_t (&n)[6], int slabs)
 {
     const size_t L = (size_t)slabs * g.mz;
     n[0] = L * g.ny * g.cux;
@@ -505,44 +500,41 @@ size_t slab_values(const Grid<P>& g, size_t (&n)[6], int slabs)
     return s;
 }
 // The stages at coarse x resolution of S slabs (L layers).
-template <typename P, typename N>
-void launch_coarse(const Refine<P>& A, size_t S, size_t L, cudaStream_t st)
+template <typename N>
+void launch_coarse(const Refine& A, size_t S, size_t L, cudaStream_t st)
 {
-    const Grid<P>& g = A.g;
+    const Grid<double>& g = A.g;
     auto grid = [](size_t threads) { return (unsigned)std::min<size_t>((threads + kThreads - 1) / kThreads, 152 * 64); };
-    k_z_split<P, N><<<grid(S * ((size_t)g.ny * g.cux + (size_t)g.cvy * g.nx)), kThreads, 0, st>>>(A);
-    k_slab_balance<P, N><<<grid(S * g.ny * g.nx), kThreads, 0, st>>>(A);
+    k_z_split<N><<<grid(S * ((size_t)g.ny * g.cux + (size_t)g.cvy * g.nx)), kThreads, 0, st>>>(A);
+    k_slab_balance<N><<<grid(S * g.ny * g.nx), kThreads, 0, st>>>(A);
     const unsigned gy = grid(L * g.ny * ((size_t)g.cux + g.nx));
-    if (g.my == 2 && !g.walls) k_y_split<P, N, true><<<gy, kThreads, 0, st>>>(A);
-    else k_y_split<P, N, false><<<gy, kThreads, 0, st>>>(A);
-    k_row_v<P, N><<<grid(L * g.cvy * g.nx), kThreads, 0, st>>>(A);
+    if (g.my == 2 && !g.walls) k_y_split<N, true><<<gy, kThreads, 0, st>>>(A);
+    else k_y_split<N, false><<<gy, kThreads, 0, st>>>(A);
+    k_row_v<N><<<grid(L * g.cvy * g.nx), kThreads, 0, st>>>(A);
 }
 
 }  // namespace
 
-template <typename P>
-int refine_slabs(const Grid<P>& g)
+int refine_slabs(const Grid<double>& g)
 {
     size_t n[6];
     int s = g.nz;
     // (and at most 65535 chunks of layers in a launch)
-    while (s > 1 && (slab_values(g, n, s) * sizeof(P) > kRefineWork || (size_t)s * g.mz > 65535u * kDenseLayers)) s = (s + 1) / 2;
+    while (s > 1 && (slab_values(g, n, s) * sizeof(double) > kRefineWork || (size_t)s * g.mz > 65535u * kDenseLayers))
+        s = (s + 1) / 2;
     return s;
 }
-template int refine_slabs<double>(const Grid<double>&);
 
-template <typename P>
-size_t refine_work(const Grid<P>& g, int slabs)
+size_t refine_work(const Grid<double>& g, int slabs)
 {
     size_t n[6];
-    return slab_values(g, n, slabs) * sizeof(P);
+    return slab_values(g, n, slabs) * sizeof(double);
 }
 
-template <typename P>
-cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, P* const out[3], P* const copy[3],
-                          unsigned* vmax, P* work, int slabs, cudaStream_t st)
+cudaError_t launch_refine(const Grid<double>& g, const double* U, const double* V, const double* W, double* const out[3], double* const copy[3],
+                          unsigned* vmax, double* work, int slabs, cudaStream_t st)
 {
-    Refine<P> A;
+    Refine A;
     A.g = g;
     A.U = U; A.V = V; A.W = W;
     A.Us = out[0]; A.Vs = out[1]; A.Ws = out[2];
@@ -550,24 +542,24 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
     A.Ve = copy ? copy[1] : nullptr;
     A.We = copy ? copy[2] : nullptr;
     A.vmax = vmax;
-    A.iDX = P(1) / g.DX;
-    A.iDY = P(1) / g.DY;
+    A.iDX = 1.0 / g.DX;
+    A.iDY = 1.0 / g.DY;
     A.dydX = g.dy / g.DX;
     A.dxdy = g.dx / g.dy;
     cudaError_t e = cudaSuccess;
     if (vmax) e = cudaMemsetAsync(vmax, 0, 3 * sizeof(unsigned), st);
     const int form = g.mx == 2 ? (g.walls ? 1 : 2) : (g.mx == 4 ? 3 : 0);
-    void (*const forms[4])(const Refine<P>) = {k_dense<P, 0, false>, k_dense<P, 2, false>, k_dense<P, 2, true>, k_dense<P, 4, false>};
-    void (*const dense)(const Refine<P>) = forms[form];
-    const int smem = (5 * kDenseRows + 2) * 32 * g.mx * (int)sizeof(P);
+    void (*const forms[4])(const Refine) = {k_dense<0, false>, k_dense<2, false>, k_dense<2, true>, k_dense<4, false>};
+    void (*const dense)(const Refine) = forms[form];
+    const int smem = (5 * kDenseRows + 2) * 32 * g.mx * (int)sizeof(double);
     static unsigned long long done[4];                     // one bit per device, for each form (mx <= 8: 84 KB in FP64)
     if (e == cudaSuccess)
-        e = smem_optin(reinterpret_cast<const void*>(dense), (5 * kDenseRows + 2) * 32 * 8 * (int)sizeof(P),
+        e = smem_optin(reinterpret_cast<const void*>(dense), (5 * kDenseRows + 2) * 32 * 8 * (int)sizeof(double),
                        &done[form]);
     if (e != cudaSuccess) return e;
     size_t n[6];
     slab_values(g, n, slabs);
-    P** const part[6] = {&A.UZ, &A.VZ, &A.WC, &A.UO, &A.WY, &A.VR};
+    double** const part[6] = {&A.UZ, &A.VZ, &A.WC, &A.UO, &A.WY, &A.VR};
     for (int q = 0; q < 6; ++q) {
         *part[q] = work;
         work += n[q];
@@ -576,8 +568,8 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
         A.K1 = std::min(A.K0 + slabs, g.nz);
         const size_t S = A.K1 - A.K0, L = S * g.mz;
         // 32-bit indexes unless a slab is enormous
-        if (slab_values(g, n, (int)S) < (1ull << 31)) launch_coarse<P, unsigned>(A, S, L, st);
-        else launch_coarse<P, size_t>(A, S, L, st);
+        if (slab_values(g, n, (int)S) < (1ull << 31)) launch_coarse<unsigned>(A, S, L, st);
+        else launch_coarse<size_t>(A, S, L, st);
         // eight layers of a column per block (one more W plane split), fewer where that
         // would leave SMs without four blocks
         const size_t tiles = (size_t)((g.nx + 31) / 32) * ((g.Ny + kDenseRows - 1) / kDenseRows);
@@ -589,9 +581,6 @@ cudaError_t launch_refine(const Grid<P>& g, const P* U, const P* V, const P* W, 
     }
     return e;
 }
-template size_t refine_work<double>(const Grid<double>&, int);
-template cudaError_t launch_refine<double>(const Grid<double>&, const double*, const double*, const double*,
-                                           double* const[3], double* const[3], unsigned*, double*, int, cudaStream_t);
 
 template <typename P>
 cudaError_t launch_refine_in_place(const Grid<P>& g, const P* U, const P* V, const P* W, P* Us, P* Vs, P* Ws, P* scrW,
