@@ -98,7 +98,9 @@ __device__ __forceinline__ long long zflux(Bal tb, Bal tt, Bal wlo, Bal whi, Bal
     return mul(bal((p.H << 3) + (p.M >> 29)), w);
 }
 
-template <int R, bool WALLS, bool LF>
+// DIFF: the diffusion of layers in FP64 arithmetic by differences (as k_step_stored has
+// it), or folded (as k_step_periodic has it: the periodic explicit form).
+template <int R, bool WALLS, bool DIFF, bool LF>
 __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
 {
     after_previous();
@@ -275,11 +277,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
         }
         if (plain) {
             // FP64 arithmetic with the same shared fluxes; the bottom faces' are
-            // carried from a layer below that was stepped in the same way.  Diffusion
-            // by differences, as k_step_stored has it, but for the periodic explicit
-            // form, which is k_step_periodic's
+            // carried from a layer below that was stepped in the same way
             const double cdn = A.zs * g.cdn[k], cup = A.zs * g.cup[k];
-            const bool folded = !WALLS && A.zs == 1.0;
             const double ndiag = -2.0 * (g.kx2 + g.ky2) - cdn - cup;
             double xt[R];
 #pragma unroll
@@ -295,28 +294,31 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
             }
             primed = false;
             carried = true;
-            double fs = s[kV * 32] * (hs + xt[0]), ds = es;
+            // ds: T^{s-1} of the row to the south (DIFF: the difference from it)
+            double fs = s[kV * 32] * (hs + xt[0]), ds = DIFF ? xd[0] - es : es;
             if (WALLS && j0 == 0) fs = 0.0;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 double fw = s[(kU + r) * 32] * (__shfl_up_sync(0xffffffffu, xt[r], 1) + xt[r]);
                 if (WALLS && !xin) fw = 0.0;
                 const double fe = __shfl_down_sync(0xffffffffu, fw, 1);
-                const double dw = __shfl_up_sync(0xffffffffu, xd[r], 1), de = __shfl_down_sync(0xffffffffu, xd[r], 1);
+                double dw = __shfl_up_sync(0xffffffffu, xd[r], 1);
+                if (DIFF) dw = xd[r] - dw;
+                const double de = __shfl_down_sync(0xffffffffu, DIFF ? dw : xd[r], 1);
                 const double tn = r + 1 < R ? xt[r + 1 < R ? r + 1 : r] : hn, dn = r + 1 < R ? xd[r + 1 < R ? r + 1 : r] : en;
                 double fn = s[(kV + r + 1) * 32] * (xt[r] + tn);
                 if (WALLS && j0 + r + 1 >= g.Ny) fn = 0.0;
                 const double ft = top ? 0.0 : s[(kW + r) * 32] * (g.wlo[k + 1] * xt[r] + g.whi[k + 1] * rt[r]);
                 const double below = k > 0 ? *at(pd - plane, ro[r + 1]) : pl;
-                const double D = folded ? g.kx2 * (dw + de) + g.ky2 * (ds + dn) + cdn * below + cup * rd[r] + ndiag * xd[r]
-                                        : g.kx2 * ((de - xd[r]) - (xd[r] - dw)) + g.ky2 * ((dn - xd[r]) - (xd[r] - ds)) +
-                                              cup * (rd[r] - xd[r]) - cdn * (xd[r] - below);
+                const double dd = DIFF ? dn - xd[r] : dn;
+                const double D = DIFF ? g.kx2 * (de - dw) + g.ky2 * (dd - ds) + cup * (rd[r] - xd[r]) - cdn * (xd[r] - below)
+                                      : g.kx2 * (dw + de) + g.ky2 * (ds + dd) + cdn * below + cup * rd[r] + ndiag * xd[r];
                 const double sum = g.hx * (fw - fe) + g.hy * (fs - fn) + g.inv_dz[k] * (__longlong_as_double(fb[r]) - ft) + D;
                 if (mine && j0 + r < g.Ny)
                     *const_cast<double*>(at(A.out + (size_t)k * plane, ro[r + 1])) =
                         LF ? fma(A.gdt, sum, xd[r]) : fma(A.gdt, sum, A.a * xd[r] + A.b * xt[r]);
                 fs = fn;
-                ds = xd[r];
+                ds = DIFF ? dd : xd[r];
                 fb[r] = __double_as_longlong(ft);
             }
         } else {
@@ -377,11 +379,14 @@ template <int R>
 cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
 {
     const Grid<double>& g = A.g;
-    void (*const k)(const Args) = g.walls ? (lf ? k_step_fix<R, true, true> : k_step_fix<R, true, false>)
-                                          : (lf ? k_step_fix<R, false, true> : k_step_fix<R, false, false>);
+    const int form = g.walls ? 2 : (A.zs != 1.0 ? 1 : 0);  // walled; periodic implicit; periodic explicit
+    void (*const forms[6])(const Args) = {k_step_fix<R, false, false, false>, k_step_fix<R, false, false, true>,
+                                          k_step_fix<R, false, true, false>,  k_step_fix<R, false, true, true>,
+                                          k_step_fix<R, true, true, false>,   k_step_fix<R, true, true, true>};
+    void (*const k)(const Args) = forms[2 * form + lf];
     constexpr int smem = kWarps * 2 * stage_rows(R) * 32 * (int)sizeof(double);
-    static unsigned long long done[4];                    // one bit per device, for each form
-    cudaError_t e = smem_optin(reinterpret_cast<const void*>(k), smem, &done[2 * (g.walls != 0) + lf]);
+    static unsigned long long done[6];                    // one bit per device, for each form
+    cudaError_t e = smem_optin(reinterpret_cast<const void*>(k), smem, &done[2 * form + lf]);
     if (e != cudaSuccess) return e;
     // The chunks of layers: as many as give the shortest run, the rounds of
     // resident blocks times the layers of a chunk, each chunk's start counted as
