@@ -206,14 +206,17 @@ __device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_
 }
 
 // Sum of T vol and of (T - mean)^2 vol (vol = dz_k, in FP64; the host applies dx dy), the
-// count of non-finite values and their sum of squares into out[0..3].  A unit takes
-// T relative to a value c near its own mean, so that its squares do not cancel;
-// thread 0 refers the units' sums to the c of the block's first one, and the block
-// that finishes last (an atomic count, nothing waits) combines the blocks' (sum,
-// squares, weight) about the common mean, in a fixed order.
-// 256 x 256 x 192 FP32 cells: 34 us (32 about one cell; 40 instructions per cell, and the last block's
-// FP64 combination at the end); a pass for the mean and one for the squares took
-// 2 x 20 us, each with a copy of the partials to the host and a synchronisation.
+// count of non-finite values and their sum of squares into out[0..3].  A block's
+// first unit takes T relative to a value near its own mean (near_mean), each further
+// one relative to the mean of the one before, so that no squares cancel beyond what
+// the differences between units add to the variance anyway; thread 0 refers the
+// units' sums to the first one's value, and the block that finishes last (an atomic
+// count, nothing waits) combines the blocks' (sum, squares, weight) about the common
+// mean, in a fixed order.
+// 256 x 256 x 192 FP32 cells: 34 us (40 instructions per cell, and the last block's
+// FP64 combination at the end; 32 us about a block's first cell, which an outlier
+// there makes useless); a pass for the mean and one for the squares took 2 x 20 us,
+// each with a copy of the partials to the host and a synchronisation.
 template <typename P>
 __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __restrict__ T, const double* __restrict__ dz,
                                                       int per_plane, double vtot, double* __restrict__ partials, 
@@ -222,15 +225,14 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
     const size_t plane = (size_t)g.Nx * g.Ny, per = (plane + per_plane - 1) / per_plane;
     const int units = g.Nz * per_plane;
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};              // thread 0: S1, S2, weight, bad, poison
-    P cb = P(0);                                          // c of the block's first unit
+    P c = P(0), cb = P(0);                                // this unit's value, the first unit's
     bool first = true;
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
         const int k = u / per_plane;
         const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
         if (lo >= hi) continue;
         const P* r = T + (size_t)k * plane;
-        const P c = near_mean(r, lo, hi);
-        if (first) cb = c;
+        if (first) c = cb = near_mean(r, lo, hi);
         first = false;
         Sum<P> s[2];
         int bad = 0;
@@ -261,6 +263,10 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
             v[3] += n[0];
             v[4] += n[1];
         }
+        // the next unit's value, in every thread alike (near this one's mean will do)
+        const float count = (float)(hi - lo) - (float)n[0];
+        const P m = c + (P)w[0] * (P)(1.0f / count);
+        c = isfinite(m) ? m : P(0);
     }
     __shared__ bool last;
     if (threadIdx.x == 0) {

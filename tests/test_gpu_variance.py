@@ -3,10 +3,14 @@ against extended-precision sums: as accurate as about the mean, wherever they li
 import numpy as np
 import pytest
 
-from tests.test_gpu_diagnostics import _case
+from tests import test_gpu_diagnostics as diagnostics
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+
+# 1700 layers of a unit each: more units than blocks
+diagnostics.SIZES.setdefault("tall", dict(nx=10, ny=4, nz=425, mx=3, my=1, mz=4, walls=0, gamma=1.1))
 
 
 def _fill(T, where, rng):
@@ -23,14 +27,16 @@ def _fill(T, where, rng):
             flat[:, q:q + per // 8] += 1e3
     elif where == "one layer":
         T[0] += 1e3
+    elif where == "alternate layers":            # among them a block's units, 1216 apart
+        T[(np.arange(Nz) // 1216) % 2 == 1] += 1e3
     return T
 
 
-@pytest.mark.parametrize("where", ["first cells", "one column", "eighths", "one layer"])
-@pytest.mark.parametrize("size", ["wide", "walls_odd"])
+@pytest.mark.parametrize("where", ["first cells", "one column", "eighths", "one layer", "alternate layers"])
+@pytest.mark.parametrize("size", ["wide", "walls_odd", "tall"])
 @pytest.mark.parametrize("f64", [True, False])
 def test_outliers_cost_no_precision(size, where, f64):
-    mr, h, d, zf, walls, W = _case(size, f64)
+    mr, h, d, zf, walls, W = diagnostics._case(size, f64)
     rng = np.random.default_rng(11)
     T = _fill(1e-3 * rng.standard_normal(h.shapes["T"]), where, rng)
     T = T if f64 else T.astype(np.float32)
