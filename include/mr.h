@@ -71,7 +71,9 @@ typedef struct {
     double ra, pr_or_sc;      /* kappa = (ra * pr_or_sc)^-1/2                  */
     double dt;                /* time step (see mr_cfl_dt / mr_set_dt)        */
     int32_t precision;        /* MR_F64: FP64 storage, flux arithmetic in FP64
-                                 or 64-bit fixed point of the same accuracy;
+                                 or, from 196,608 cells, 64-bit fixed point of
+                                 the same accuracy relative to the largest
+                                 values around a cell;
                                  MR_F32: FP32 storage and flux arithmetic.
                                  Reductions are of FP64 accuracy in both.     */
     int32_t velocity_mode;    /* MR_VEL_STORED: dense faces kept in HBM;

@@ -19,8 +19,8 @@
 //
 // Measured on 256 x 256 x 192 cells (coarse 128 x 128 x 96): 0.212 ms per step,
 // 2.8 TB/s on the 48 B/cell of the method; 0.597 ms with one thread per cell and
-// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  About 325
-// instructions per cell issue at 0.56 per clock and scheduler; integer
+// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  366 instructions
+// per cell (of a warp, times 32) issue at 0.59 per clock and scheduler; integer
 // multiply-adds and the integer ALU share the time, so what bounds it is the
 // decoding (14 instructions a value, 6.7 values a cell) and the 46 multiply-adds.
 // Rows: 3 per warp 0.214 ms, 4 (12 instead of 16 warps per SM) 0.225, 2 (two
@@ -41,12 +41,17 @@
 // (and not all zero), or which holds an infinity, a NaN or only values near the
 // underflow limit, is stepped in FP64 arithmetic instead (22 operations per cell:
 // a field that falls off by many decades from cell to cell everywhere runs at
-// 0.71 ms, one of zeros and ones at 0.30 ms).  So is every layer where gdt 2^eR
+// 0.72 ms, 0.79 to 0.81 on walled or implicit grids, one of zeros and ones at
+// 0.29 ms).  So is every layer where gdt 2^eR
 // exceeds 2^kMaxRate = 64: a stable explicit step's rates are below 16 (2^eR is up
 // to four times their sum), and beyond the limit the products' error, 2^-58 of
 // them, would pass FP64's rounding -- a single face velocity far above all others
 // with a time step that follows the others, or implicit vertical diffusion over
 // layers much thinner than the time step needs.
+// So a result is as accurate as FP64 arithmetic's relative to the largest values
+// around its cell, not to its own value where that is much smaller; and as decoding
+// and products round down, stepping -T gives the negatives to rounding only (an ulp
+// of the largest value; exactly odd rounding would cost 10 % of a step).
 #include <math.h>
 
 #include "mr_fix.cuh"
@@ -302,23 +307,32 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
                 double fw = s[(kU + r) * 32] * (__shfl_up_sync(0xffffffffu, xt[r], 1) + xt[r]);
                 if (WALLS && !xin) fw = 0.0;
                 const double fe = __shfl_down_sync(0xffffffffu, fw, 1);
-                double dw = __shfl_up_sync(0xffffffffu, xd[r], 1);
-                if (DIFF) dw = xd[r] - dw;
-                const double de = __shfl_down_sync(0xffffffffu, DIFF ? dw : xd[r], 1);
+                double dx;                                // the two x neighbours (DIFF: the second difference)
+                if constexpr (DIFF) {
+                    dx = xd[r] - __shfl_up_sync(0xffffffffu, xd[r], 1);
+                    dx = __shfl_down_sync(0xffffffffu, dx, 1) - dx;
+                } else {
+                    dx = __shfl_up_sync(0xffffffffu, xd[r], 1) + __shfl_down_sync(0xffffffffu, xd[r], 1);
+                }
                 const double tn = r + 1 < R ? xt[r + 1 < R ? r + 1 : r] : hn, dn = r + 1 < R ? xd[r + 1 < R ? r + 1 : r] : en;
                 double fn = s[(kV + r + 1) * 32] * (xt[r] + tn);
                 if (WALLS && j0 + r + 1 >= g.Ny) fn = 0.0;
                 const double ft = top ? 0.0 : s[(kW + r) * 32] * (g.wlo[k + 1] * xt[r] + g.whi[k + 1] * rt[r]);
                 const double below = k > 0 ? *at(pd - plane, ro[r + 1]) : pl;
-                const double dd = DIFF ? dn - xd[r] : dn;
-                const double D = DIFF ? g.kx2 * (de - dw) + g.ky2 * (dd - ds) + cup * (rd[r] - xd[r]) - cdn * (xd[r] - below)
-                                      : g.kx2 * (dw + de) + g.ky2 * (ds + dd) + cdn * below + cup * rd[r] + ndiag * xd[r];
+                double D;
+                if constexpr (DIFF) {
+                    const double dd = dn - xd[r];
+                    D = g.kx2 * dx + g.ky2 * (dd - ds) + cup * (rd[r] - xd[r]) - cdn * (xd[r] - below);
+                    ds = dd;
+                } else {
+                    D = g.kx2 * dx + g.ky2 * (ds + dn) + cdn * below + cup * rd[r] + ndiag * xd[r];
+                    ds = xd[r];
+                }
                 const double sum = g.hx * (fw - fe) + g.hy * (fs - fn) + g.inv_dz[k] * (__longlong_as_double(fb[r]) - ft) + D;
                 if (mine && j0 + r < g.Ny)
                     *const_cast<double*>(at(A.out + (size_t)k * plane, ro[r + 1])) =
                         LF ? fma(A.gdt, sum, xd[r]) : fma(A.gdt, sum, A.a * xd[r] + A.b * xt[r]);
                 fs = fn;
-                ds = DIFF ? dd : xd[r];
                 fb[r] = __double_as_longlong(ft);
             }
         } else {
@@ -410,9 +424,18 @@ cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
 }  // namespace
 
 // Grids it takes: 32-bit byte offsets inside a plane, second-order faces, and at
-// least 196,608 cells.  Below that too few warps march too long a chain, and one
-// thread per cell in FP64 arithmetic (mr_step.cu) is as fast: 14.5 us per step
-// both ways on 64 x 64 x 48 cells, 8.4 us here against 6.3 us on 32 x 32 x 32.
+// least 196,608 cells.  On small grids too few warps march too long a chain, and one
+// thread per cell in FP64 arithmetic (mr_step.cu) is as fast or faster.  us per step
+// here and there, M = 2, steps back to back:
+//   cells      periodic        walled          implicit z (either)
+//   32,768     5.5    3.1      5.7    4.9      12.3   12.3
+//   69,120     7.2    6.8      7.0   10.7      14.4   18.5
+//   110,592   10.4   12.4     10.4   13.8      16.4   22.6
+//   153,088   10.5   12.3     10.5   13.8      18.5   22.6
+//   196,608   14.9   12.4     14.9   25.8      20.4   28.7
+//   317,440   15.2   21.5     15.0   34.9      24.6   47.2
+// The line is where periodic explicit grids cross for good, and it is one for all
+// forms; walled and implicit grids would gain from about 50,000 cells on.
 bool step_fix_fits(const Grid<double>& g)
 {
     const size_t row = (size_t)(g.ufx > g.Nx ? g.ufx : g.Nx), rows = (size_t)(g.vfy > g.Ny ? g.vfy : g.Ny);
