@@ -19,7 +19,7 @@
 //
 // Measured on 256 x 256 x 192 cells (coarse 128 x 128 x 96): 0.212 ms per step,
 // 2.8 TB/s on the 48 B/cell of the method; 0.597 ms with one thread per cell and
-// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  366 instructions
+// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  367 instructions
 // per cell (of a warp, times 32) issue at 0.59 per clock and scheduler; integer
 // multiply-adds and the integer ALU share the time, so what bounds it is the
 // decoding (14 instructions a value, 6.7 values a cell) and the 46 multiply-adds.
