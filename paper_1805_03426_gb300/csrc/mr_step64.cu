@@ -41,7 +41,7 @@
 // (and not all zero), or which holds an infinity, a NaN or only values near the
 // underflow limit, is stepped in FP64 arithmetic instead (22 operations per cell:
 // a field that falls off by many decades from cell to cell everywhere runs at
-// 0.72 ms, 0.79 to 0.81 on walled or implicit grids, one of zeros and ones at
+// 0.65 ms, 0.74 to 0.78 on walled or implicit grids, one of zeros and ones at
 // 0.29 ms).  So is every layer where gdt 2^eR
 // exceeds 2^kMaxRate = 64: a stable explicit step's rates are below 16 (2^eR is up
 // to four times their sum), and beyond the limit the products' error, 2^-58 of
@@ -80,6 +80,12 @@ struct LayerK {
     Bal wlo, whi;                    // weights of the layer's top face, times 2^62
 };
 
+// And what a layer in FP64 arithmetic takes: 1 / dz, the vertical rates, the diagonal,
+// the weights of the top face.
+struct LayerP {
+    double iz, cdn, cup, ndiag, wlo, whi;
+};
+
 struct Args {
     Grid<double> g;
     const double *U, *V, *W, *Tm1, *T;
@@ -112,6 +118,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
     let_next();
     const Grid<double>& g = A.g;
     __shared__ LayerK sk[kMaxChunk];
+    __shared__ LayerP sp[kMaxChunk];
     __shared__ Bal sc[4];                                 // 4 S_U hx, 4 S_V hy, kx2, ky2
     const int k0 = blockIdx.y * A.kc, k1 = min(k0 + A.kc, g.Nz);
     const int lane = threadIdx.x & 31;
@@ -130,6 +137,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
                          4.0 * (g.kx2 + g.ky2);
         eR = exponent(r);                                 // 2^eR > r
         usable = usable && eR > -400 && eR < 400 && exponent(A.gdt) + eR <= kMaxRate;
+    }
+    for (int q = threadIdx.x - 64; q >= 0 && q < k1 - k0; q += blockDim.x) {   // (other warps' lanes than below)
+        const int k = k0 + q;
+        const double cdn = A.zs * g.cdn[k], cup = A.zs * g.cup[k];
+        sp[q] = LayerP{g.inv_dz[k], cdn, cup, -2.0 * (g.kx2 + g.ky2) - cdn - cup, g.wlo[k + 1], g.whi[k + 1]};
     }
     if (usable) {
         for (int q = threadIdx.x; q < k1 - k0; q += blockDim.x) {
@@ -283,8 +295,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
         if (plain) {
             // FP64 arithmetic with the same shared fluxes; the bottom faces' are
             // carried from a layer below that was stepped in the same way
-            const double cdn = A.zs * g.cdn[k], cup = A.zs * g.cup[k];
-            const double ndiag = -2.0 * (g.kx2 + g.ky2) - cdn - cup;
+            const LayerP& L = sp[k - k0];
             double xt[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -317,18 +328,18 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_step_fix(const Args A)
                 const double tn = r + 1 < R ? xt[r + 1 < R ? r + 1 : r] : hn, dn = r + 1 < R ? xd[r + 1 < R ? r + 1 : r] : en;
                 double fn = s[(kV + r + 1) * 32] * (xt[r] + tn);
                 if (WALLS && j0 + r + 1 >= g.Ny) fn = 0.0;
-                const double ft = top ? 0.0 : s[(kW + r) * 32] * (g.wlo[k + 1] * xt[r] + g.whi[k + 1] * rt[r]);
+                const double ft = top ? 0.0 : s[(kW + r) * 32] * (L.wlo * xt[r] + L.whi * rt[r]);
                 const double below = k > 0 ? *at(pd - plane, ro[r + 1]) : pl;
-                double D;
+                double sum;
                 if constexpr (DIFF) {
                     const double dd = dn - xd[r];
-                    D = g.kx2 * dx + g.ky2 * (dd - ds) + cup * (rd[r] - xd[r]) - cdn * (xd[r] - below);
+                    sum = g.kx2 * dx + g.ky2 * (dd - ds) + L.cup * (rd[r] - xd[r]) - L.cdn * (xd[r] - below);
                     ds = dd;
                 } else {
-                    D = g.kx2 * dx + g.ky2 * (ds + dn) + cdn * below + cup * rd[r] + ndiag * xd[r];
+                    sum = g.kx2 * dx + g.ky2 * (ds + dn) + L.cdn * below + L.cup * rd[r] + L.ndiag * xd[r];
                     ds = xd[r];
                 }
-                const double sum = g.hx * (fw - fe) + g.hy * (fs - fn) + g.inv_dz[k] * (__longlong_as_double(fb[r]) - ft) + D;
+                sum = fma(L.iz, __longlong_as_double(fb[r]) - ft, fma(g.hy, fs - fn, fma(g.hx, fw - fe, sum)));
                 if (mine && j0 + r < g.Ny)
                     *const_cast<double*>(at(A.out + (size_t)k * plane, ro[r + 1])) =
                         LF ? fma(A.gdt, sum, xd[r]) : fma(A.gdt, sum, A.a * xd[r] + A.b * xt[r]);
