@@ -540,9 +540,10 @@ cudaError_t launch_adj_step(const Grid<P>& g, const P* Us, const P* Vs, const P*
                                     Tprev, Mn, Mc, Mp, s_nu, s_var, mean_prev, gU, gV, gW, (P)c.a, (P)c.b, (P)c.gdt, cx, cy,
                                     cz, march);
         }
-        return launch_after(euler ? k_adj_step_periodic<P, true> : k_adj_step_periodic<P, false>, grd, blk, 0, st, g, Us, Vs,
-                            Ws, T, Tprev, Mn, Mc, Mp, s_nu, s_var, mean_prev, gU, gV, gW, (P)c.a, (P)c.b, (P)c.gdt, cx, cy,
-                            cz);
+        const auto k = euler ? k_adj_step_periodic<P, true> : k_adj_step_periodic<P, false>;
+        const bool ahead = sizeof(P) == 4 || fp64_gains_ahead(reinterpret_cast<const void*>(k), grd, 256);
+        return launch_after_if(ahead, k, grd, blk, 0, st, g, Us, Vs, Ws, T, Tprev, Mn, Mc, Mp, s_nu, s_var, mean_prev, gU, gV,
+                               gW, (P)c.a, (P)c.b, (P)c.gdt, cx, cy, cz);
     }
     if (euler)
         k_adj_step<P, true><<<grd, blk, 0, st>>>(g, Us, Vs, Ws, T, Tprev, Mn, Mc, Mp, s_nu, s_var, mean_prev, gU, gV,

@@ -25,7 +25,7 @@ namespace mr {
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... K, typename... A>
-cudaError_t launch_after(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+cudaError_t launch_after_if(bool ahead, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -36,9 +36,24 @@ cudaError_t launch_after(void (*kernel)(K...), dim3 grid, dim3 block, size_t sme
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ahead ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
+template <typename... K, typename... A>
+cudaError_t launch_after(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+{
+    return launch_after_if(true, kernel, grid, block, smem, st, args...);
+}
+// Whether a kernel bound by the FP64 pipe gains from an early start.  Its blocks come
+// up where the step before leaves room: where two grids fit on the chip at once, on
+// every SM alike; where they do not, on the SMs that empty first, and the pipes of the
+// others idle, step after step.  From three quarters of the resident blocks on
+// there are enough of them to even out.  us per step ahead and not, 152 SMs:
+// periodic (912 resident blocks) 440 blocks 6.8 and 8.3, 480 12.3 and 10.3, 598 12.3
+// and 10.3, 782 12.5 and 14.4; fourth order (608) 288 blocks 9.0 and 10.3, 360 16.7 and
+// 14.4, 440 16.6 and 14.4, 480 16.8 and 18.5; walls (1216) 598 blocks 13.8 and 16.4, 720
+// 25.8 and 18.5.
+bool fp64_gains_ahead(const void* kernel, dim3 grid, int threads);
 
 constexpr int kPlateBlocks = 304;  // blocks of the plate Nusselt reduction
 constexpr int kMomentBlocks = 152 * 8;   // blocks of the volume moments

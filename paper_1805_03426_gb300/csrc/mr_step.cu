@@ -5,6 +5,9 @@
 // C = -(1/Vol) sum_faces u_f T_f A_f (outward), D = (1/Vol) sum kappa A dT/dn.
 // Per-layer coefficients (1/dz, interpolation weights, kappa/(dz d)) come
 // from the handle's grid, so a stretched z costs no extra arithmetic.
+#include <mutex>
+#include <unordered_map>
+
 #include "mr_internal.cuh"
 
 namespace mr {
@@ -33,8 +36,7 @@ struct FaceVel {
 // f-2 .. f+1 at T[base + c * stride] with the grid's weights; periodic cells
 // wrap, cells beyond a wall carry zero weight and are not read.
 template <typename P>
-__device__ __forceinline__ P face4(const P* w, int f, int N, bool periodic, const P* T,
-                                   size_t base, size_t stride)
+__device__ __forceinline__ P face4(const P* w, int f, int N, bool periodic, const P* T, size_t base, size_t stride)
 {
     P s = 0;
 #pragma unroll
@@ -51,12 +53,9 @@ __device__ __forceinline__ P face4(const P* w, int f, int N, bool periodic, cons
 // (D_z(T^{s-1}) + plate terms) / 2; the implicit half follows in k_zsolve.
 // O4: fourth-order face values of the advected scalar.
 template <typename P, bool IMPLZ, bool LERP, bool O4>
-__global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P, LERP> Us,
-                                                     const FaceVel<P, LERP> Vs, const FaceVel<P, LERP> Ws,
-                                                     const P* Tm1, const P* T, P* __restrict__ Tp1, P a, P b, P gdt)
+__device__ __forceinline__ void step_cell(const Grid<P>& g, const FaceVel<P, LERP>& Us, const FaceVel<P, LERP>& Vs,
+                                          const FaceVel<P, LERP>& Ws, const P* Tm1, const P* T, P* Tp1, P a, P b, P gdt)
 {
-    after_previous();
-    let_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
@@ -124,6 +123,15 @@ __global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P,
     const P C = cx * g.inv_dx + cy * g.inv_dy + cz * g.inv_dz[k];
     const P D = g.kx2 * dx_ + g.ky2 * dy_ + dz_;
     Tp1[m] = a * Dc + b * Tc + gdt * (C + D);
+}
+template <typename P, bool IMPLZ, bool LERP, bool O4>
+__global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P, LERP> Us, const FaceVel<P, LERP> Vs,
+                                                     const FaceVel<P, LERP> Ws, const P* Tm1, const P* T,
+                                                     P* __restrict__ Tp1, P a, P b, P gdt)
+{
+    after_previous();
+    let_next();
+    step_cell<P, IMPLZ, LERP, O4>(g, Us, Vs, Ws, Tm1, T, Tp1, a, b, gdt);
 }
 
 // The same step (Eq. 5) for the common case -- periodic x and y, explicit
@@ -405,12 +413,15 @@ cudaError_t step_stored(const Grid<P>& g, const FaceVel<P, LERP>& u, const FaceV
                                     dim3((unsigned)((quads + 127) / 128), (unsigned)layers), 128, 0, st, g, u.A, v.A, w.A,
                                     Tm1, T, Tp1, a, b, gdt, march);
         }
-        return launch_after(c.a == 1.0 && c.b == 0.0 ? k_step_periodic<P, true> : k_step_periodic<P, false>, grd, blk, 0, st,
-                            g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
+        const auto k = c.a == 1.0 && c.b == 0.0 ? k_step_periodic<P, true> : k_step_periodic<P, false>;
+        const bool ahead = sizeof(P) == 4 || fp64_gains_ahead(reinterpret_cast<const void*>(k), grd, 256);
+        return launch_after_if(ahead, k, grd, blk, 0, st, g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
     }
-    return launch_after(g.order4 ? (implz ? k_step_stored<P, true, LERP, true> : k_step_stored<P, false, LERP, true>)
-                                 : (implz ? k_step_stored<P, true, LERP, false> : k_step_stored<P, false, LERP, false>),
-                        grd, blk, 0, st, g, u, v, w, Tm1, T, Tp1, a, b, gdt);
+    // (with implicit z the solve lies between the steps)
+    const auto k = g.order4 ? (implz ? k_step_stored<P, true, LERP, true> : k_step_stored<P, false, LERP, true>)
+                            : (implz ? k_step_stored<P, true, LERP, false> : k_step_stored<P, false, LERP, false>);
+    const bool ahead = sizeof(P) == 4 || implz || fp64_gains_ahead(reinterpret_cast<const void*>(k), grd, 256);
+    return launch_after_if(ahead, k, grd, blk, 0, st, g, u, v, w, Tm1, T, Tp1, a, b, gdt);
 }
 
 __global__ void k_lerp(const float* A, const float* B, float alpha, float* __restrict__ out,
@@ -432,6 +443,27 @@ cudaError_t launch_lerp_f32(const float* A, const float* B, double alpha, float*
     const size_t want = (n + 255) / 256;
     const unsigned blocks = (unsigned)(want < 152 * 16 ? want : 152 * 16);
     return launch_after(k_lerp, blocks, 256, 0, st, A, B, (float)alpha, out, n);
+}
+
+bool fp64_gains_ahead(const void* kernel, dim3 grid, int threads)
+{
+    static std::mutex mu;
+    static std::unordered_map<const void*, int> resident;     // blocks per SM
+    int r = 0;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        const auto it = resident.find(kernel);
+        if (it != resident.end()) {
+            r = it->second;
+        } else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, threads, 0) == cudaSuccess) {
+            resident[kernel] = r;
+        } else {
+            cudaGetLastError();
+            return true;
+        }
+    }
+    const size_t blocks = (size_t)grid.x * grid.y * grid.z, slots = (size_t)152 * r;
+    return 2 * blocks <= slots || 4 * blocks > 3 * slots;
 }
 
 template <typename P>

@@ -33,7 +33,7 @@ def test_kernels_launched_ahead_declare_no_read_only_inputs():
 def test_every_kernel_launched_ahead_waits():
     names = set()
     for f in glob.glob(os.path.join(CSRC, "*.cu")):
-        for call in re.findall(r"launch_after\((.*?)\);", open(f).read(), flags=re.S):
+        for call in re.findall(r"(?:launch_after(?:_if)?\(|const auto k =)(.*?);", open(f).read(), flags=re.S):
             names |= set(re.findall(r"\bk_\w+", call))
     waits = {n for n, _, body in _kernels() if "after_previous()" in body}
     assert names and names <= waits, names - waits
