@@ -15,6 +15,7 @@ namespace {
 
 constexpr double kTBottom = 0.5;
 constexpr double kTTop = -0.5;
+constexpr size_t kAloneCells = (size_t)4 << 20;
 
 // Dense face velocity of a step: one stored field, or (LERP) the linear
 // interpolation A + alpha (B - A) between the fields of two coarse time
@@ -131,6 +132,15 @@ __global__ void __launch_bounds__(256) k_step_stored(Grid<P> g, const FaceVel<P,
 {
     after_previous();
     let_next();
+    step_cell<P, IMPLZ, LERP, O4>(g, Us, Vs, Ws, Tm1, T, Tp1, a, b, gdt);
+}
+// Not launched ahead, so that the scalar is read-only while it lives and may be loaded
+// as such.
+template <typename P, bool IMPLZ, bool LERP, bool O4>
+__global__ void __launch_bounds__(256) k_step_stored_alone(Grid<P> g, const FaceVel<P, LERP> Us, const FaceVel<P, LERP> Vs,
+                                                           const FaceVel<P, LERP> Ws, const P* __restrict__ Tm1,
+                                                           const P* __restrict__ T, P* __restrict__ Tp1, P a, P b, P gdt)
+{
     step_cell<P, IMPLZ, LERP, O4>(g, Us, Vs, Ws, Tm1, T, Tp1, a, b, gdt);
 }
 
@@ -416,6 +426,16 @@ cudaError_t step_stored(const Grid<P>& g, const FaceVel<P, LERP>& u, const FaceV
         const auto k = c.a == 1.0 && c.b == 0.0 ? k_step_periodic<P, true> : k_step_periodic<P, false>;
         const bool ahead = sizeof(P) == 4 || fp64_gains_ahead(reinterpret_cast<const void*>(k), grd, 256);
         return launch_after_if(ahead, k, grd, blk, 0, st, g, u.A, v.A, w.A, Tm1, T, Tp1, a, b, gdt);
+    }
+    if constexpr (sizeof(P) == 4) {
+        // FP32 at fourth order: from 4 M cells on read-only loads gain more than an early
+        // start, which does not allow them (us per step: 3.1 M cells 63.5 and 62.7,
+        // 4.2 M 84.2 and 87.5, 16.8 M 638 and 683)
+        if (g.order4 && (size_t)g.Nx * g.Ny * g.Nz >= kAloneCells) {
+            (implz ? k_step_stored_alone<P, true, LERP, true> : k_step_stored_alone<P, false, LERP, true>)
+                <<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
+            return cudaGetLastError();
+        }
     }
     // (with implicit z the solve lies between the steps)
     const auto k = g.order4 ? (implz ? k_step_stored<P, true, LERP, true> : k_step_stored<P, false, LERP, true>)

@@ -1,5 +1,6 @@
 """Steps on both sides of the rules that choose how a step is launched, against the
-oracle: FP64 grids whose blocks fit the chip twice, once and more often."""
+oracle: FP64 grids whose blocks fit the chip twice, once and more often, fourth-order
+FP32 grids from 4 M cells (their own kernel) and below."""
 import numpy as np
 import pytest
 
@@ -54,3 +55,13 @@ def test_fp64_backward_steps(mr, n):
     _, gr = _oracle_grad(p, 9, *w)
     for a, b in zip(g, gr):
         assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+
+
+# 160 x 160 x 160 cells and 160 x 166 x 160 (4.10 M, 4.25 M; the rule's 4 M is 4,194,304)
+@pytest.mark.parametrize("ny", [80, 83])
+@pytest.mark.parametrize("form", [dict(), dict(walls=1), dict(implicit=1)])
+def test_fourth_order_fp32_steps(mr, ny, form):
+    p = Problem(80, ny, 80, gamma=1.2, dt=2e-4, ra=1e7, np_average=4, face_order=4, **form)
+    assert (p.T0.size >= 4 << 20) == (ny == 83)
+    _, ref = O.run(p.cfg, O.refine(p.cfg, p.U, p.V, p.W), p.T0, 5)
+    assert np.abs(_run(mr, p, mr.MR_F32, 5) - ref).max() <= 1e-5
