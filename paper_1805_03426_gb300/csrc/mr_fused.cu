@@ -1350,7 +1350,13 @@ cudaError_t launch_fused_plate_nu(const Grid<float>& g, const float* T, double i
     const size_t plane = (size_t)g.Nx * g.Ny;
     const size_t want = (plane + kCRThreads * kCRCells - 1) / (kCRThreads * kCRCells);
     const unsigned blocks = 2 * (unsigned)std::min(want, (size_t)kCRNu);
-    return launch_after(k_coupled_nu, blocks, kCRThreads, 0, st, T, plane, (size_t)(g.Nz - 1) * plane, izb, izt,
+    // Ahead of its time on the smallest and on large planes: of some dozens or hundreds of
+    // blocks that come up beside the step's last CTAs several share an SM's FP64 pipe (us
+    // per coupled step ahead and not: 64 x 64 cells a plate 11.6 and 12.7, 128 x 128 25.0
+    // and 18.8, 320 x 144 50.7 and 45.2, 384 x 384 133 and 127, 512 x 384 234 and 230,
+    // 512 x 512 288 and 293, 1024 x 1024 381 and 392).
+    const bool ahead = plane < (1u << 13) || plane >= (1u << 18);
+    return launch_after_if(ahead, k_coupled_nu, blocks, kCRThreads, 0, st, T, plane, (size_t)(g.Nz - 1) * plane, izb, izt,
                         1.0 / (double)plane, work, nu2);
 }
 

@@ -1,6 +1,6 @@
 """Steps on both sides of the rules that choose how a step is launched, against the
 oracle: FP64 grids whose blocks fit the chip twice, once and more often, fourth-order
-FP32 grids from 4 M cells (their own kernel) and below."""
+FP32 grids from 4 M cells (their own kernel) and below, coupled steps over plate sizes."""
 import numpy as np
 import pytest
 
@@ -65,3 +65,19 @@ def test_fourth_order_fp32_steps(mr, ny, form):
     assert (p.T0.size >= 4 << 20) == (ny == 83)
     _, ref = O.run(p.cfg, O.refine(p.cfg, p.U, p.V, p.W), p.T0, 5)
     assert np.abs(_run(mr, p, mr.MR_F32, 5) - ref).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n", [(32, 16, 8), (64, 32, 8), (256, 256, 4)])
+def test_coupled_steps_over_plate_sizes(mr, n):
+    p = Problem(*n, gamma=1.2, dt=2e-4, ra=1e7)
+    h = mr.mr_create(p.mr_config(mr, mr.MR_F32, mr.MR_VEL_FUSED))
+    nu = torch.zeros(2, dtype=torch.float64, device="cuda")
+    Tc = torch.zeros((n[2], n[1], n[0]), dtype=torch.float64, device="cuda")
+    mr.mr_set_scalar(h, dev(p.T0))
+    for _ in range(3):
+        mr.mr_refine_velocity(h, dev(p.U), dev(p.V), dev(p.W))
+        mr.mr_scalar_step_coupled(h, nu, Tc)
+    st = mr.mr_scalar_stats(h)
+    for k, name in enumerate(("nu_bot", "nu_top")):
+        assert abs(float(nu[k]) - st[name]) <= 1e-12 * abs(st[name])
+    h.close()
