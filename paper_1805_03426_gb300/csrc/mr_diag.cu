@@ -166,15 +166,17 @@ __device__ __forceinline__ void moments_unit(const P* __restrict__ r, size_t lo,
 
 // A value near the mean of a unit, in every thread: the mean of kGroup samples per
 // thread spread over it (finite ones; 0 without any).  Whatever the samples miss or
-// hit, the squares about it are at most units / samples (8) times those about the
-// unit's mean, so that at most three bits of them cancel; about one cell's value an
-// outlier just there would cost as many bits as the unit has.
+// hit, the squares about it are at most cells / samples (16) times those about the
+// unit's mean, so that at most four bits of them cancel; about one cell's value an
+// outlier just there would cost as many bits as the unit has.  The sum's last steps
+// are one thread's and the division is FP32's: FP64 operations are dear.
 template <typename P>
 __device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_t hi)
 {
-    constexpr int kGroup = 8;
+    constexpr int kGroup = 4;
     __shared__ P sum[kThreads / 32];
     __shared__ int num[kThreads / 32];
+    __shared__ P mean;
     const size_t step = (hi - lo) / kGroup;
     P s = P(0);
     int n = 0;
@@ -194,15 +196,16 @@ __device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_
         num[threadIdx.x >> 5] = n;
     }
     __syncthreads();
-    s = P(0);
-    n = 0;
-    for (int w = 0; w < kThreads / 32; ++w) {
-        s += sum[w];
-        n += num[w];
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kThreads / 32; ++w) {
+            s += sum[w];
+            n += num[w];
+        }
+        const P c = s * (P)(1.0f / (float)(n > 0 ? n : 1));
+        mean = isfinite(c) ? c : P(0);
     }
-    __syncthreads();                                      // sum, num are reused
-    const P c = s / P(n > 0 ? n : 1);
-    return isfinite(c) ? c : P(0);
+    __syncthreads();
+    return mean;
 }
 
 // Sum of T vol and of (T - mean)^2 vol (vol = dz_k, in FP64; the host applies dx dy), the
