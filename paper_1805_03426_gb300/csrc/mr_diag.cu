@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
             v[4] += n[1];
         }
         // the next unit's value, in every thread alike (near this one's mean will do)
+        if (u + (int)gridDim.x >= units) break;
         const float count = (float)(hi - lo) - (float)n[0];
         const P m = c + (P)w[0] * (P)(1.0f / count);
         c = isfinite(m) ? m : P(0);

@@ -430,7 +430,7 @@ cudaError_t step_stored(const Grid<P>& g, const FaceVel<P, LERP>& u, const FaceV
     if constexpr (sizeof(P) == 4) {
         // FP32 at fourth order: from 4 M cells on read-only loads gain more than an early
         // start, which does not allow them (us per step: 3.1 M cells 63.5 and 62.7,
-        // 4.2 M 84.2 and 87.5, 16.8 M 638 and 683)
+        // 4.2 M 84.2 and 87.5, 33.6 M 638 and 683)
         if (g.order4 && (size_t)g.Nx * g.Ny * g.Nz >= kAloneCells) {
             (implz ? k_step_stored_alone<P, true, LERP, true> : k_step_stored_alone<P, false, LERP, true>)
                 <<<grd, blk, 0, st>>>(g, u, v, w, Tm1, T, Tp1, a, b, gdt);
