@@ -136,22 +136,38 @@ __device__ __forceinline__ void block_sum(Sum<A> (&v)[NV], double (&out)[NV])
 
 // ------------------------------------------------------------- moments
 
+// Whether a value is finite, and whether it is NaN; FP64 ones from their bits, a
+// comparison taking as long as an addition.
+__device__ __forceinline__ bool finite(float t) { return isfinite(t); }
+__device__ __forceinline__ bool finite(double t) { return ((unsigned)__double2hiint(t) & 0x7ff00000u) != 0x7ff00000u; }
+__device__ __forceinline__ bool is_nan(float t) { return isnan(t); }
+__device__ __forceinline__ bool is_nan(double t)
+{
+    const unsigned hi = (unsigned)__double2hiint(t) & 0x7fffffffu;
+    return hi > 0x7ff00000u || (hi == 0x7ff00000u && __double2loint(t) != 0);
+}
+// The sum of squares of values that are not finite, of which some are NaN (2) or not (1).
+__device__ __forceinline__ double squares_of(int poison)
+{
+    return __hiloint2double(poison & 2 ? 0x7ff80000 : (poison ? 0x7ff00000 : 0), 0);
+}
+
 // One unit of a plane: sum and sum of squares of T - c over its finite values,
-// their number's complement (bad), the sum of squares of the others (infinite or
-// NaN), and the largest magnitude.
+// their number's complement (bad), what the others are (squares_of), and the
+// largest magnitude.
 template <typename A, typename P>
 __device__ __forceinline__ void moments_unit(const P* __restrict__ r, size_t lo, size_t hi, P c, Sum<A>& s1, Sum<A>& s2,
-                                             int& bad, P& poison, P& big)
+                                             int& bad, int& poison, P& big)
 {
     constexpr int kGroup = 8;                              // loads in flight
     size_t m = lo + threadIdx.x;
     auto one = [&](P t) {
-        if (isfinite(t)) {
-            big = fmax(big, fabs(t));
+        if (finite(t)) {
+            if constexpr (sizeof(P) == 4) big = fmaxf(big, fabsf(t));
             s1.diff(t, c, s2);
         } else {
             ++bad;
-            poison += t * t;
+            poison |= is_nan(t) ? 2 : 1;
         }
     };
     for (; m + (kGroup - 1) * kThreads < hi; m += kGroup * kThreads) {
@@ -164,31 +180,34 @@ __device__ __forceinline__ void moments_unit(const P* __restrict__ r, size_t lo,
     for (; m < hi; m += kThreads) one(r[m]);
 }
 
-// A value near the mean of a unit, in every thread: the mean of kGroup samples per
-// thread spread over it (finite ones; 0 without any).  Whatever the samples miss or
-// hit, the squares about it are at most cells / samples (16) times those about the
-// unit's mean, so that at most four bits of them cancel; about one cell's value an
-// outlier just there would cost as many bits as the unit has.  The sum's last steps
-// are one thread's and the division is FP32's: FP64 operations are dear.
+// A value near the mean of one or more units: kSample samples per thread and unit,
+// spread over it (finite ones), and their mean in every thread (0 without any).
+// Whatever the samples miss or hit, the squares about it are at most cells / samples
+// (16) times those about the units' mean, so that at most four bits of them cancel;
+// about one cell's value an outlier just there would cost as many bits as the units
+// have.  The sum's last steps are one thread's and the division is FP32's: FP64
+// operations are dear.
+constexpr int kSample = 4;
 template <typename P>
-__device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_t hi)
+__device__ __forceinline__ void sample(const P* __restrict__ r, size_t lo, size_t hi, P& s, int& n)
 {
-    constexpr int kGroup = 4;
-    __shared__ P sum[kThreads / 32];
-    __shared__ int num[kThreads / 32];
-    __shared__ P mean;
-    const size_t step = (hi - lo) / kGroup;
-    P s = P(0);
-    int n = 0;
+    const size_t step = (hi - lo) / kSample;
 #pragma unroll
-    for (int q = 0; q < kGroup; ++q) {
+    for (int q = 0; q < kSample; ++q) {
         const size_t m = lo + q * step + threadIdx.x;
         const P t = m < hi ? r[m] : P(NAN);
-        if (isfinite(t)) {
+        if (finite(t)) {
             s += t;
             ++n;
         }
     }
+}
+template <typename P>
+__device__ __forceinline__ P sample_mean(P s, int n)
+{
+    __shared__ P sum[kThreads / 32];
+    __shared__ int num[kThreads / 32];
+    __shared__ P mean;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     n = __reduce_add_sync(0xffffffffu, n);
     if ((threadIdx.x & 31) == 0) {
@@ -209,13 +228,17 @@ __device__ __forceinline__ P near_mean(const P* __restrict__ r, size_t lo, size_
 }
 
 // Sum of T vol and of (T - mean)^2 vol (vol = dz_k, in FP64; the host applies dx dy), the
-// count of non-finite values and their sum of squares into out[0..3].  A block's
-// first unit takes T relative to a value near its own mean (near_mean), each further
-// one relative to the mean of the one before, so that no squares cancel beyond what
-// the differences between units add to the variance anyway; thread 0 refers the
-// units' sums to the first one's value, and the block that finishes last (an atomic
-// count, nothing waits) combines the blocks' (sum, squares, weight) about the common
-// mean, in a fixed order.
+// count of non-finite values and their sum of squares into out[0..3].  An FP32 block's
+// first unit takes T relative to a value near its own mean, each further one relative
+// to the mean of the one before, so that no squares cancel beyond what the
+// differences between units add to the variance anyway; every unit's pairs are summed
+// over the block, and thread 0 refers them to the first one's value.  An FP64 block
+// takes one value near the mean of all its units, and its threads add up their own
+// sums until the end: the FP64 pipe bounds it, three operations a cell (512 x 512 x 256
+// cells: 469 us for the statistics, 771 with the units summed over the block one by
+// one and FP64 comparisons, 682 in two passes).  The block that finishes last (an
+// atomic count, nothing waits) combines the blocks' (sum, squares, weight) about the
+// common mean, in a fixed order.
 // 256 x 256 x 192 FP32 cells: 34 us (40 instructions per cell, and the last block's
 // FP64 combination at the end; 32 us about a block's first cell, which an outlier
 // there makes useless); a pass for the mean and one for the squares took 2 x 20 us,
@@ -229,48 +252,83 @@ __global__ void __launch_bounds__(kThreads) k_moments(Grid<P> g, const P* __rest
     const int units = g.Nz * per_plane;
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};              // thread 0: S1, S2, weight, bad, poison
     P c = P(0), cb = P(0);                                // this unit's value, the first unit's
-    bool first = true;
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
-        const int k = u / per_plane;
-        const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
-        if (lo >= hi) continue;
-        const P* r = T + (size_t)k * plane;
-        if (first) c = cb = near_mean(r, lo, hi);
-        first = false;
-        Sum<P> s[2];
-        int bad = 0;
-        P poison = P(0), big = fabs(c);
-        moments_unit(r, lo, hi, c, s[0], s[1], bad, poison, big);
-        double w[2];
-        if (__syncthreads_or(!in_range(big, kLeastT))) {
+    if constexpr (sizeof(P) == 8) {
+        P s = P(0);
+        int n = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+            const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
+            if (lo < hi) sample(T + (size_t)(u / per_plane) * plane, lo, hi, s, n);
+        }
+        cb = sample_mean(s, n);
+        Sum<double> a[5];
+        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+            const int k = u / per_plane;
+            const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
+            if (lo >= hi) continue;
             Sum<double> d[2];
-            bad = 0;
-            poison = P(0);
-            moments_unit(r, lo, hi, c, d[0], d[1], bad, poison, big);
-            block_sum(d, w);
-        } else {
-            block_sum(s, w);
+            int bad = 0, poison = 0;
+            P big = P(0);
+            moments_unit(T + (size_t)k * plane, lo, hi, cb, d[0], d[1], bad, poison, big);
+            const double z = dz[k];
+            a[0].s = fma(d[0].s, z, a[0].s);
+            a[1].s = fma(d[1].s, z, a[1].s);
+            if (threadIdx.x == 0) a[2].s = fma((double)(hi - lo), z, a[2].s);
+            if (bad) {                                    // the weight less the bad values'
+                a[2].s -= (double)bad * z;
+                a[3].s += (double)bad;
+                a[4].s += squares_of(poison);
+            }
         }
-        double n[2] = {0.0, 0.0};
-        if (__syncthreads_or(bad)) {
-            Sum<double> d[2];
-            d[0].s = (double)bad;
-            d[1].s = (double)poison;
-            block_sum(d, n);
+        block_sum(a, v);
+    } else {
+        bool first = true;
+        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+            const int k = u / per_plane;
+            const size_t lo = (size_t)(u % per_plane) * per, hi = lo + per < plane ? lo + per : plane;
+            if (lo >= hi) continue;
+            const P* r = T + (size_t)k * plane;
+            if (first) {
+                P s = P(0);
+                int n = 0;
+                sample(r, lo, hi, s, n);
+                c = cb = sample_mean(s, n);
+            }
+            first = false;
+            Sum<P> s[2];
+            int bad = 0, poison = 0;
+            P big = fabs(c);
+            moments_unit(r, lo, hi, c, s[0], s[1], bad, poison, big);
+            double w[2];
+            if (__syncthreads_or(!in_range(big, kLeastT))) {
+                Sum<double> d[2];
+                bad = 0;
+                poison = 0;
+                moments_unit(r, lo, hi, c, d[0], d[1], bad, poison, big);
+                block_sum(d, w);
+            } else {
+                block_sum(s, w);
+            }
+            double n[2] = {0.0, 0.0};
+            if (__syncthreads_or(bad)) {
+                Sum<double> d[2];
+                d[0].s = (double)bad;
+                d[1].s = squares_of(poison);
+                block_sum(d, n);
+            }
+            if (threadIdx.x == 0) {
+                const double good = (double)(hi - lo) - n[0], d = (double)c - (double)cb;
+                v[0] = fma(fma(d, good, w[0]), dz[k], v[0]);
+                v[1] = fma(fma(d, fma(d, good, 2.0 * w[0]), w[1]), dz[k], v[1]);
+                v[2] = fma(good, dz[k], v[2]);
+                v[3] += n[0];
+                v[4] += n[1];
+            }
+            // the next unit's value, in every thread alike (near this one's mean will do)
+            if (u + (int)gridDim.x >= units) break;
+            const float count = (float)(hi - lo) - (float)n[0];
+            const P m = c + (P)w[0] * (P)(1.0f / count);
+            c = isfinite(m) ? m : P(0);
         }
-        if (threadIdx.x == 0) {
-            const double good = (double)(hi - lo) - n[0], d = (double)c - (double)cb;
-            v[0] = fma(fma(d, good, w[0]), dz[k], v[0]);
-            v[1] = fma(fma(d, fma(d, good, 2.0 * w[0]), w[1]), dz[k], v[1]);
-            v[2] = fma(good, dz[k], v[2]);
-            v[3] += n[0];
-            v[4] += n[1];
-        }
-        // the next unit's value, in every thread alike (near this one's mean will do)
-        if (u + (int)gridDim.x >= units) break;
-        const float count = (float)(hi - lo) - (float)n[0];
-        const P m = c + (P)w[0] * (P)(1.0f / count);
-        c = isfinite(m) ? m : P(0);
     }
     __shared__ bool last;
     if (threadIdx.x == 0) {
