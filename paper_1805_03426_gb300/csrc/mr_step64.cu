@@ -17,9 +17,9 @@
 // and accumulates  sum rates x (flux differences, diffusion neighbours)  in one
 // wide integer, which the FP64 pipe then scales and adds to T^{s-1}.
 //
-// Measured on 256 x 256 x 192 cells (coarse 128 x 128 x 96): 0.212 ms per step,
-// 2.8 TB/s on the 48 B/cell of the method; 0.597 ms with one thread per cell and
-// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  367 instructions
+// Measured on 256 x 256 x 192 cells (coarse 128 x 128 x 96): 0.210 ms per step,
+// 2.9 TB/s on the 48 B/cell of the method; 0.597 ms with one thread per cell and
+// 25 FP64 operations per cell, which ran the FP64 pipe at 88 %.  365 instructions
 // per cell (of a warp, times 32) issue at 0.59 per clock and scheduler; integer
 // multiply-adds and the integer ALU share the time, so what bounds it is the
 // decoding (14 instructions a value, 6.7 values a cell) and the 46 multiply-adds.
@@ -441,9 +441,9 @@ cudaError_t launch_r(Args& A, bool lf, cudaStream_t st)
 //   cells      periodic        walled          implicit z (either)
 //   32,768     5.5    3.1      5.7    4.9      12.3   12.3
 //   69,120     7.2    6.8      7.0   10.7      14.4   18.5
-//   110,592   10.4   12.4     10.4   13.8      16.4   22.6
-//   153,088   10.5   12.3     10.5   13.8      18.5   22.6
-//   196,608   14.9   12.4     14.9   25.8      20.4   28.7
+//   110,592   10.4   10.3     10.4   13.8      16.4   22.6
+//   153,088   10.5   10.3     10.5   13.8      18.5   22.6
+//   196,608   14.9   12.4     14.9   21.9      20.4   28.7
 //   317,440   15.2   21.5     15.0   34.9      24.6   47.2
 // The line is where periodic explicit grids cross for good, and it is one for all
 // forms; walled and implicit grids would gain from about 50,000 cells on.
